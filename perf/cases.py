@@ -33,7 +33,7 @@ def listed():
         # the Sod shock tube at its own resolution, in the precision it is validated in: the smallest calls
         _case("sod_400x4_fp64", "sod", 400, 4, "fp64", 100, sides="tube", mu=3e-6),
         # disturbed thermal Couette flow between plates, run for very many steps: a thin grid with wall sides
-        _case("couette_2x100_fp32", "couette", 2, 100, "fp32", 200, sides="plates", sigma=0.9, mu=0.1),
+        _case("couette_2x100_fp32", "couette", 2, 100, "fp32", 200, sides="plates", sigma=0.9, mu=0.03),
         # one training pair of the surrogate: random smooth field, 16 steps
         _case("fourier_256_fp32", "fourier", 256, 256, "fp32", 16, mu=1e-4),
         # the convected vortex on the grid the method is quoted on, fields out every 100 steps, and its validation in FP64
