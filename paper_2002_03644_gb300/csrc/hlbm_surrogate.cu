@@ -16,8 +16,8 @@
 //
 // Weight gradient: dW[co][ci][tap] = sum_pixels dz[pixel, co] *
 // h[pixel + offset(tap), ci], a GEMM over pixels on the tensor cores
-// (BF16 operands, FP32 accumulators), added to the FP32 gradient with
-// atomics.
+// (BF16 operands, FP32 accumulators) whose partial sums are added up in a
+// fixed order.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -340,134 +340,423 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t b[4], const void *p)
                  : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(a));
 }
 
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+{
+    const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem));
+}
+// 16 bytes, or zeros where !valid (gmem is not read then)
+__device__ __forceinline__ void cp_async16_or_zero(void *smem, const void *gmem, bool valid)
+{
+    const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "r"(valid ? 16 : 0));
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::); }
+__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 // Weight gradient on the tensor cores: for one tap, dW[co][ci] += sum over
 // pixels p of dz[p, co] h[p + off(tap), ci], a GEMM with the pixels as its
-// K dimension (M = output channels, N = input channels).  BF16 tiles of dz
-// and of the shifted activations ([pixel][channel], rows padded by 8 for
-// conflict-free ldmatrix) are staged in shared memory and read transposed
-// into the A and B fragments of mma.sync m16n8k16; each of the 4 warps
-// accumulates a 32 x 32 block of the (at most) 64 x 64 result in FP32 over
-// its CTA's pixel chunk, then adds it to the FP32 gradient (real channels
-// only).  The bias gradient (tap 4 CTAs) sums the FP32 dz.  One CTA per
-// (chunk, tap).
-constexpr int WG_THREADS = 128, WG_KC = 64;
+// K dimension (M = output channels, N = input channels).  One CTA computes
+// CIB input channels of one tap over a chunk of WG_CHUNK pixels: BF16 tiles
+// of dz and of the shifted activations ([pixel][channel], rows padded by 8
+// for conflict-free ldmatrix) stream through a ring of WG_STAGES shared-
+// memory stages of WG_KC pixels (cp.async, so that a stage's copy overlaps
+// the products of the ones before it) and are read transposed into the A
+// and B fragments of mma.sync m16n8k16.  A thread keeps the image position
+// of each pixel it copies and advances it by WG_KC per stage, so that any
+// image width works without a division; two warps only copy, so that this
+// arithmetic does not stand in the chains of the products.  A result's FP32 chain runs over
+// the chunk's pixels in order, and every CTA's sums go to its own slice of
+// `part`, which wgrad_reduce_kernel adds up in a fixed order.
+constexpr int WG_KC = 64, WG_STAGES = 4, WG_CHUNK = 16384;
 
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(WG_THREADS)
-wgrad_mma_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ dzb,
-                 const float *__restrict__ dzf, int cin, int cout, int npix, int H, int W, int chunk,
-                 float *__restrict__ dW, float *__restrict__ db)
+template <int COUT, int CIB>
+struct WgGeom {
+    static constexpr int M16 = COUT / 16, N16 = CIB / 16;  // 16 x 16 blocks of the result
+    // warps along the rows and columns of the result
+    static constexpr bool SQ = M16 % 2 == 0 && N16 % 2 == 0;
+    static constexpr int WN = SQ ? 2 : (N16 % 4 == 0 ? 4 : (M16 % 4 == 0 || M16 == 3 ? 1 : N16));
+    static constexpr int WM = SQ ? 2 : (N16 % 4 == 0 ? 1 : (M16 % 4 == 0 ? 4 : (M16 == 3 ? 3 : (N16 == 3 ? 1 : M16))));
+    static constexpr int MT = M16 / WM, NT = N16 / WN;  // blocks per warp
+    static constexpr int MMA_WARPS = WM * WN, COPIERS = 64;
+    static constexpr int THREADS = 32 * MMA_WARPS + COPIERS;
+    static constexpr int LDA = COUT + 8, LDB = CIB + 8;
+    static constexpr int STAGE = WG_KC * (LDA + LDB);
+    static constexpr size_t smem_bytes = (size_t)WG_STAGES * STAGE * sizeof(__nv_bfloat16);
+    static_assert(M16 % WM == 0 && N16 % WN == 0, "whole blocks per warp");
+};
+
+// grid: (chunk, tap, block of CIB input channels)
+template <int CIN, int COUT, int CIB>
+__global__ void __launch_bounds__(WgGeom<COUT, CIB>::THREADS)
+wgrad_mma_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ dzb, int npix, int H, int W,
+                 float *__restrict__ part)
 {
-    constexpr int LDA = COUT + 8, LDB = CIN + 8;
-    constexpr int MT = COUT / 16, NTT = CIN / 8;
-    constexpr int CA = COUT / 8, CB = CIN / 8;  // 16-byte chunks per staged row
-    __shared__ __align__(16) __nv_bfloat16 sA[WG_KC * LDA];
-    __shared__ __align__(16) __nv_bfloat16 sB[WG_KC * LDB];
-    const int tap = blockIdx.y;
-    const int dp = tap / 3 - 1, dq = tap % 3 - 1;
-    const int p0 = blockIdx.x * chunk;
-    const int p1 = min(p0 + chunk, npix);
-    const int HW = H * W;
+    using G = WgGeom<COUT, CIB>;
+    constexpr int CA = COUT / 8, CB = CIB / 8;  // 16-byte pieces per pixel
+    constexpr int LDA = G::LDA, LDB = G::LDB, MT = G::MT, NT = G::NT;
+    constexpr int NA = WG_KC * CA / G::COPIERS, NB = WG_KC * CB / G::COPIERS;  // copies per copying thread
+    extern __shared__ __align__(16) unsigned char wg_smem[];
+    __nv_bfloat16 *ring = reinterpret_cast<__nv_bfloat16 *>(wg_smem);  // [stage][KC][LDA], [KC][LDB]
+    const int tap = blockIdx.y, dp = tap / 3 - 1, dq = tap % 3 - 1, c0 = blockIdx.z * CIB;
+    const int p0 = blockIdx.x * WG_CHUNK, p1 = min(p0 + WG_CHUNK, npix);
+    const int nstage = (p1 - p0 + WG_KC - 1) / WG_KC;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t4 = lane & 3, lj = lane >> 3, lr = lane & 7;
-    const int mt0 = 2 * (warp >> 1), nt0 = 4 * (warp & 1);
-    float acc[2][4][4];
+    const int m0 = (warp % G::WM) * MT * 16, n0 = (warp / G::WM) * NT * 16;
+    const bool copier = warp >= G::MMA_WARPS;
+    const int ct = threadIdx.x - 32 * G::MMA_WARPS;
+
+    // the pixels of this thread's copies of h: column, row, first pixel of the image
+    int pj[NB], pi[NB], pn[NB];
 #pragma unroll
-    for (int i = 0; i < 2; i++)
+    for (int e = 0; e < NB; e++) {
+        const int p = p0 + (copier ? ct + e * G::COPIERS : 0) / CB, row = p / W;
+        pj[e] = p - row * W;
+        pi[e] = row % H;
+        pn[e] = (row - pi[e]) * W;
+    }
+    auto load = [&](int k) {  // stage k: pixels p0 + KC k ..
+        __nv_bfloat16 *sA = ring + (k % WG_STAGES) * G::STAGE, *sB = sA + WG_KC * LDA;
+        const int q0 = p0 + k * WG_KC;
 #pragma unroll
-        for (int j = 0; j < 4; j++)
+        for (int e = 0; e < NA; e++) {
+            const int x = ct + e * G::COPIERS, r = x / CA, c8 = x - r * CA;
+            cp_async16_or_zero(sA + r * LDA + c8 * 8, dzb + (size_t)(q0 + r) * COUT + c8 * 8, q0 + r < p1);
+        }
+#pragma unroll
+        for (int e = 0; e < NB; e++) {
+            const int x = ct + e * G::COPIERS, r = x / CB, c8 = x - r * CB;
+            const bool in = q0 + r < p1;
+            const size_t src = in ? (size_t)pn[e] + (size_t)wrap(pi[e] + dp, H) * W + wrap(pj[e] + dq, W) : 0;
+            cp_async16_or_zero(sB + r * LDB + c8 * 8, h + src * CIN + c0 + c8 * 8, in);
+            pj[e] += WG_KC;
+            while (pj[e] >= W) {
+                pj[e] -= W;
+                if (++pi[e] == H) { pi[e] = 0; pn[e] += H * W; }
+            }
+        }
+    };
+    float acc[MT][2 * NT][4];
+#pragma unroll
+    for (int i = 0; i < MT; i++)
+#pragma unroll
+        for (int j = 0; j < 2 * NT; j++)
 #pragma unroll
             for (int k = 0; k < 4; k++) acc[i][j][k] = 0.0f;
-    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-    for (int q0 = p0; q0 < p1; q0 += WG_KC) {
-        __syncthreads();  // the previous sub-chunk's fragments are read
-        for (int e = threadIdx.x; e < WG_KC * CA; e += WG_THREADS) {
-            const int r = e / CA, c8 = e - r * CA;
-            const int p = q0 + r;
-            *reinterpret_cast<uint4 *>(sA + r * LDA + c8 * 8) =
-                p < p1 ? *reinterpret_cast<const uint4 *>(dzb + (size_t)p * COUT + c8 * 8) : zero;
+#pragma unroll
+    for (int k = 0; k < WG_STAGES - 1; k++) {
+        if (copier && k < nstage) load(k);
+        cp_async_commit();
+    }
+    for (int k = 0; k < nstage; k++) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(WG_STAGES - 2) : "memory");
+        __syncthreads();  // stage k has arrived; stage k - 1 is read
+        if (copier) {
+            if (k + WG_STAGES - 1 < nstage) load(k + WG_STAGES - 1);
+            cp_async_commit();
+            continue;
         }
-        for (int e = threadIdx.x; e < WG_KC * CB; e += WG_THREADS) {
-            const int r = e / CB, c8 = e - r * CB;
-            const int p = q0 + r;
-            uint4 v = zero;
-            if (p < p1) {
-                const int n = p / HW, rem = p - n * HW, i = rem / W, j = rem - i * W;
-                const int src = n * HW + wrap(i + dp, H) * W + wrap(j + dq, W);
-                v = *reinterpret_cast<const uint4 *>(h + (size_t)src * CIN + c8 * 8);
-            }
-            *reinterpret_cast<uint4 *>(sB + r * LDB + c8 * 8) = v;
-        }
-        __syncthreads();
+        const __nv_bfloat16 *sA = ring + (k % WG_STAGES) * G::STAGE, *sB = sA + WG_KC * LDA;
 #pragma unroll
         for (int k0 = 0; k0 < WG_KC; k0 += 16) {
-            uint32_t a[2][4];
+            uint32_t a[MT][4], b[NT][4];
 #pragma unroll
-            for (int mi = 0; mi < 2; mi++)
-                if (mt0 + mi < MT)
-                    ldsm_x4_t(a[mi], sA + (k0 + (lj >> 1) * 8 + lr) * LDA + (mt0 + mi) * 16 + (lj & 1) * 8);
+            for (int i = 0; i < MT; i++)
+                ldsm_x4_t(a[i], sA + (k0 + (lj >> 1) * 8 + lr) * LDA + m0 + i * 16 + (lj & 1) * 8);
 #pragma unroll
-            for (int ni = 0; ni < 4; ni += 2) {
-                if (nt0 + ni + 1 < NTT) {
-                    uint32_t b[4];
-                    ldsm_x4_t(b, sB + (k0 + (lj & 1) * 8 + lr) * LDB + (nt0 + ni) * 8 + (lj >> 1) * 8);
+            for (int j = 0; j < NT; j++)
+                ldsm_x4_t(b[j], sB + (k0 + (lj & 1) * 8 + lr) * LDB + n0 + j * 16 + (lj >> 1) * 8);
 #pragma unroll
-                    for (int mi = 0; mi < 2; mi++) {
-                        if (mt0 + mi < MT) {
-                            mma_bf16(acc[mi][ni], a[mi], b);
-                            mma_bf16(acc[mi][ni + 1], a[mi], b + 2);
-                        }
-                    }
+            for (int i = 0; i < MT; i++)
+#pragma unroll
+                for (int j = 0; j < NT; j++) {
+                    mma_bf16(acc[i][2 * j], a[i], b[j]);
+                    mma_bf16(acc[i][2 * j + 1], a[i], b[j] + 2);
+                }
+        }
+    }
+    if (copier) return;
+    float *dst = part + ((size_t)blockIdx.x * 9 + tap) * COUT * CIN;
+#pragma unroll
+    for (int i = 0; i < MT; i++)
+#pragma unroll
+        for (int j = 0; j < 2 * NT; j++)
+#pragma unroll
+            for (int r = 0; r < 2; r++) {
+                const int co = m0 + i * 16 + g + 8 * r, ci = c0 + n0 + j * 8 + 2 * t4;
+                *reinterpret_cast<float2 *>(dst + (size_t)co * CIN + ci) = make_float2(acc[i][j][2 * r], acc[i][j][2 * r + 1]);
+            }
+}
+
+// The same sums with all nine taps in one CTA, for images of KT columns where
+// a chunk is whole image rows.  wgrad_mma_kernel reads dz and h once per tap,
+// and at 8 x 256^2 those 1.2 GB per 64 -> 64 layer come from L2 at 4.6 TB/s
+// (262 us).  Here a CTA takes 16 input and COB output channels
+// of a chunk: one image row of dz at a time against the three rows of h its
+// taps reach (a ring of four row slots, the next row copied while this one
+// is computed), 96 or 128 bytes per pixel instead of nine times 256.  Warp
+// (dp, m) holds the three taps of row offset dp (a dz fragment serves three
+// taps); two more warps only copy, so that the address arithmetic of the
+// copies does not stand in the chains of the products.  The chain of a result runs over the chunk's pixels in the same
+// order as in wgrad_mma_kernel, so both give the same bits.  At 8 x 256^2 the
+// 64 -> 64 layer takes 128 us, 300 TFLOP/s: 256 CTAs, two per SM, bound by
+// their ldmatrix reads of shared memory (four per six MMAs, 12 warps: 192
+// cycles per 16-pixel step).
+template <int COUT, int KT>
+struct WgRowGeom {
+    static constexpr int COB = COUT % 32 == 0 ? 32 : 16;
+    static constexpr int LDA = COB + 8, LDB = 16 + 8;  // padded rows: conflict-free ldmatrix
+    static constexpr int MMA_WARPS = 3 * (COB / 16), COPIERS = 64;
+    static constexpr int THREADS = 32 * MMA_WARPS + COPIERS;
+    static constexpr int H_SLOT = (KT + 2) * LDB, Z_SLOT = KT * LDA;
+    static constexpr size_t smem_bytes = (size_t)(4 * H_SLOT + 2 * Z_SLOT) * sizeof(__nv_bfloat16);
+};
+
+// grid: (chunk, block of COB output channels, block of 16 input channels)
+template <int CIN, int COUT, int KT>
+__global__ void __launch_bounds__(WgRowGeom<COUT, KT>::THREADS)
+wgrad_rows_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ dzb, int nrow, int H,
+                  float *__restrict__ part)
+{
+    using G = WgRowGeom<COUT, KT>;
+    constexpr int LDA = G::LDA, LDB = G::LDB, CA = G::COB / 8;
+    extern __shared__ __align__(16) unsigned char wg_smem[];
+    __nv_bfloat16 *sH = reinterpret_cast<__nv_bfloat16 *>(wg_smem);  // [4][KT + 2][LDB]
+    __nv_bfloat16 *sZ = sH + 4 * G::H_SLOT;                          // [2][KT][LDA]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, t4 = lane & 3, lj = lane >> 3, lr = lane & 7;
+    const int o0 = blockIdx.y * G::COB, c0 = blockIdx.z * 16;
+    const int dp = warp % 3, m0 = warp / 3 * 16;
+    const bool copier = warp >= G::MMA_WARPS;
+    const int ct = threadIdx.x - 32 * G::MMA_WARPS;
+    const int r0 = blockIdx.x * (WG_CHUNK / KT), r1 = min(r0 + WG_CHUNK / KT, nrow);  // image rows n H + i
+    auto load_h = [&](int row, int slot) {  // pixels -1 .. KT (wrapped) of an image row
+        const __nv_bfloat16 *src = h + (size_t)row * KT * CIN + c0;
+        __nv_bfloat16 *dst = sH + slot * G::H_SLOT;
+        for (int e = ct; e < (KT + 2) * 2; e += G::COPIERS) {
+            const int px = e >> 1, c8 = e & 1;
+            cp_async16(dst + px * LDB + c8 * 8, src + (size_t)((px + KT - 1) % KT) * CIN + c8 * 8);
+        }
+    };
+    auto load_z = [&](int row, int buf) {
+        const __nv_bfloat16 *src = dzb + (size_t)row * KT * COUT + o0;
+        __nv_bfloat16 *dst = sZ + buf * G::Z_SLOT;
+        for (int e = ct; e < KT * CA; e += G::COPIERS) {
+            const int px = e / CA, c8 = e - px * CA;
+            cp_async16(dst + px * LDA + c8 * 8, src + (size_t)px * COUT + c8 * 8);
+        }
+    };
+    float acc[3][2][4];
+#pragma unroll
+    for (int t = 0; t < 3; t++)
+#pragma unroll
+        for (int n = 0; n < 2; n++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) acc[t][n][k] = 0.0f;
+
+    int base = 0, i = r0 % H;  // ring slot of row i - 1; the row's place in its image
+    for (int row = r0; row < r1; row++) {
+        const int buf = (row - r0) & 1;
+        const bool more = row + 1 < r1, same = i + 1 < H;
+        if (row == r0 || i == 0) base = 0;
+        if (copier) {
+            if (row == r0 || i == 0) {
+                // the first row of the chunk or of an image: fill the ring
+                load_h(i == 0 ? row + H - 1 : row - 1, 0);
+                load_h(row, 1);
+                load_h(same ? row + 1 : row - H + 1, 2);
+                if (row == r0) load_z(row, buf);
+                cp_async_commit();
+            }
+            cp_async_wait0();
+        }
+        __syncthreads();  // this row's data are in; the slots of the last row are free
+        if (copier) {
+            if (more) {
+                if (same) load_h(i + 2 < H ? row + 2 : row + 2 - H, (base + 3) & 3);
+                load_z(row + 1, buf ^ 1);
+                cp_async_commit();
+            }
+        } else {
+            const __nv_bfloat16 *A = sZ + buf * G::Z_SLOT + ((lj >> 1) * 8 + lr) * LDA + m0 + (lj & 1) * 8;
+            const __nv_bfloat16 *B = sH + ((base + dp) & 3) * G::H_SLOT + ((lj & 1) * 8 + lr) * LDB + (lj >> 1) * 8;
+#pragma unroll 4
+            for (int k0 = 0; k0 < KT; k0 += 16) {
+                uint32_t a[4], b[3][4];
+                ldsm_x4_t(a, A + k0 * LDA);
+#pragma unroll
+                for (int dq = 0; dq < 3; dq++) ldsm_x4_t(b[dq], B + (k0 + dq) * LDB);
+#pragma unroll
+                for (int dq = 0; dq < 3; dq++) {
+                    mma_bf16(acc[dq][0], a, b[dq]);
+                    mma_bf16(acc[dq][1], a, b[dq] + 2);
                 }
             }
         }
+        if (more && !same) __syncthreads();  // the next image refills the ring
+        base = (base + 1) & 3;
+        i = same ? i + 1 : 0;
     }
+    if (copier) return;
+    float *dst = part + (size_t)blockIdx.x * 9 * COUT * CIN;
 #pragma unroll
-    for (int mi = 0; mi < 2; mi++) {
+    for (int dq = 0; dq < 3; dq++)
 #pragma unroll
-        for (int ni = 0; ni < 4; ni++) {
-            if (mt0 + mi >= MT || nt0 + ni >= NTT) continue;
+        for (int n = 0; n < 2; n++)
 #pragma unroll
-            for (int r = 0; r < 2; r++)
+            for (int r = 0; r < 2; r++) {
+                const int co = o0 + m0 + g + 8 * r, ci = c0 + n * 8 + 2 * t4;
+                *reinterpret_cast<float2 *>(dst + ((size_t)(dp * 3 + dq) * COUT + co) * CIN + ci) =
+                    make_float2(acc[dq][n][2 * r], acc[dq][n][2 * r + 1]);
+            }
+}
+
+// dW[co][ci][tap] += the sum over `np` slices of part[slice][tap][co][ci]
+// (padded extents co_pad, ci_pad).  Eight threads share an output: slices
+// k, k + 8, .. each, then in order.
+__global__ void __launch_bounds__(256)
+wgrad_reduce_kernel(const float *__restrict__ part, int np, int cout, int cin, int cout_pad, int cin_pad,
+                    float *__restrict__ dW)
+{
+    __shared__ float red[8][32];
+    const int n = 9 * cout_pad * cin_pad;
+    const int e = blockIdx.x * 32 + (threadIdx.x & 31), k = threadIdx.x >> 5;
+    float sum = 0.0f;
+    if (e < n)
+#pragma unroll 4
+        for (int q = k; q < np; q += 8) sum += part[(size_t)q * n + e];
+    red[k][threadIdx.x & 31] = sum;
+    __syncthreads();
+    if (k == 0 && e < n) {
 #pragma unroll
-                for (int e = 0; e < 2; e++) {
-                    const int co = (mt0 + mi) * 16 + g + 8 * r, ci = (nt0 + ni) * 8 + 2 * t4 + e;
-                    if (co < cout && ci < cin) atomicAdd(&dW[((size_t)co * cin + ci) * 9 + tap], acc[mi][ni][2 * r + e]);
-                }
-        }
-    }
-    if (tap == 4 && (int)threadIdx.x < cout) {
-        float bacc = 0.0f;
-        for (int p = p0; p < p1; p++) bacc += dzf[(size_t)p * COUT + threadIdx.x];
-        atomicAdd(&db[threadIdx.x], bacc);
+        for (int q = 1; q < 8; q++) sum += red[q][threadIdx.x];
+        const int tap = e / (cout_pad * cin_pad), rem = e - tap * cout_pad * cin_pad;
+        const int co = rem / cin_pad, ci = rem - co * cin_pad;
+        if (co < cout && ci < cin) dW[((size_t)co * cin + ci) * 9 + tap] += sum;
     }
 }
 
-template <int CIN>
-cudaError_t launch_wgrad_cin(int cout_pad, const __nv_bfloat16 *h, const __nv_bfloat16 *dzb, const float *dzf, int cin,
-                             int cout, int npix, int H, int W, float *dW, float *db, cudaStream_t st)
+// Column sums of an FP32 [npix][C] array (the bias gradient): one partial
+// row per block, read in 16-byte pieces.
+__global__ void __launch_bounds__(256)
+colsum_kernel(const float *__restrict__ x, int C, int npix, float *__restrict__ bpart)
 {
-    const int chunk = 16384;
-    dim3 grid((npix + chunk - 1) / chunk, 9);
-    switch (cout_pad) {
-    case 16: wgrad_mma_kernel<CIN, 16><<<grid, WG_THREADS, 0, st>>>(h, dzb, dzf, cin, cout, npix, H, W, chunk, dW, db); break;
-    case 32: wgrad_mma_kernel<CIN, 32><<<grid, WG_THREADS, 0, st>>>(h, dzb, dzf, cin, cout, npix, H, W, chunk, dW, db); break;
-    case 48: wgrad_mma_kernel<CIN, 48><<<grid, WG_THREADS, 0, st>>>(h, dzb, dzf, cin, cout, npix, H, W, chunk, dW, db); break;
-    case 64: wgrad_mma_kernel<CIN, 64><<<grid, WG_THREADS, 0, st>>>(h, dzb, dzf, cin, cout, npix, H, W, chunk, dW, db); break;
-    default: return cudaErrorInvalidValue;
+    __shared__ float4 red[256];
+    const int c4 = C / 4, rows = 256 / c4;
+    const int r = threadIdx.x / c4, c = threadIdx.x - r * c4;
+    float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (r < rows) {
+#pragma unroll 4
+        for (long long p = (long long)blockIdx.x * rows + r; p < npix; p += (long long)gridDim.x * rows) {
+            const float4 v = reinterpret_cast<const float4 *>(x)[p * c4 + c];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
     }
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (r == 0) {
+        for (int q = 1; q < rows; q++) {
+            const float4 v = red[q * c4 + c];
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        }
+        reinterpret_cast<float4 *>(bpart + (size_t)blockIdx.x * C)[c] = s;
+    }
+}
+
+// db[c] += the sum over `nb` rows of bpart[row][C]: one warp per channel
+__global__ void bias_reduce_kernel(const float *__restrict__ bpart, int nb, int C, float *__restrict__ db)
+{
+    float s = 0.0f;
+    for (int q = threadIdx.x; q < nb; q += 32) s += bpart[(size_t)q * C + blockIdx.x];
+    for (int w = 16; w > 0; w >>= 1) s += __shfl_down_sync(0xffffffffu, s, w);
+    if (threadIdx.x == 0) db[blockIdx.x] += s;
+}
+
+constexpr int BIAS_BLOCKS = 304;  // partial rows of a bias gradient, at most
+
+int sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 152;
+    return n;
+}
+
+struct WgradArgs {
+    const __nv_bfloat16 *h, *dzb;
+    int cin, cout, npix, H, W;
+    float *dW, *part;  // part: one padded [9][co][ci] slice per chunk of WG_CHUNK pixels
+};
+
+template <int CIN, int COUT, int CIB>
+cudaError_t launch_wgrad_block(const WgradArgs &a, cudaStream_t st)
+{
+    using G = WgGeom<COUT, CIB>;
+    const cudaError_t e = cudaFuncSetAttribute(wgrad_mma_kernel<CIN, COUT, CIB>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem_bytes);
+    if (e != cudaSuccess) return e;
+    const int chunks = (a.npix + WG_CHUNK - 1) / WG_CHUNK;
+    wgrad_mma_kernel<CIN, COUT, CIB><<<dim3(chunks, 9, CIN / CIB), G::THREADS, G::smem_bytes, st>>>(a.h, a.dzb, a.npix,
+                                                                                                  a.H, a.W, a.part);
+    wgrad_reduce_kernel<<<(9 * CIN * COUT + 31) / 32, 256, 0, st>>>(a.part, chunks, a.cout, a.cin, COUT, CIN, a.dW);
     return cudaGetLastError();
 }
 
+template <int CIN, int COUT, int KT>
+cudaError_t launch_wgrad_rows(const WgradArgs &a, cudaStream_t st)
+{
+    using G = WgRowGeom<COUT, KT>;
+    const cudaError_t e = cudaFuncSetAttribute(wgrad_rows_kernel<CIN, COUT, KT>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::smem_bytes);
+    if (e != cudaSuccess) return e;
+    const int chunks = (a.npix + WG_CHUNK - 1) / WG_CHUNK;
+    wgrad_rows_kernel<CIN, COUT, KT><<<dim3(chunks, COUT / G::COB, CIN / 16), G::THREADS, G::smem_bytes, st>>>(
+        a.h, a.dzb, a.npix / KT, a.H, a.part);
+    wgrad_reduce_kernel<<<(9 * CIN * COUT + 31) / 32, 256, 0, st>>>(a.part, chunks, a.cout, a.cin, COUT, CIN, a.dW);
+    return cudaGetLastError();
+}
+
+// Images of 256 columns take the kernel with all taps per CTA (64 -> 64
+// channels, 8 / 4 / 1 images: 128 / 80 / 79 us against 262 / 158 / 95 us for
+// one CTA per tap; with 128 columns it was no faster, 118 against 102 us,
+// because a row is then only 8 of its steps).  Elsewhere one CTA per (chunk,
+// tap) takes all input channels where that gives 1.5 CTAs per SM, else
+// blocks of fewer channels (8 images of 128^2: 102 us).
+template <int CIN, int COUT>
+cudaError_t launch_wgrad_t(const WgradArgs &a, cudaStream_t st)
+{
+    if (a.W == 256) return launch_wgrad_rows<CIN, COUT, 256>(a, st);
+    const long long chunks = (a.npix + WG_CHUNK - 1) / WG_CHUNK, sms = sm_count();
+    const long long ctas = 9 * chunks, want = 3 * sms / 2;
+    if constexpr (CIN == 64) {
+        if (ctas < want) return 2 * ctas < want ? launch_wgrad_block<CIN, COUT, 16>(a, st) : launch_wgrad_block<CIN, COUT, 32>(a, st);
+    } else if constexpr (CIN > 16) {
+        if (ctas < want) return launch_wgrad_block<CIN, COUT, 16>(a, st);
+    }
+    return launch_wgrad_block<CIN, COUT, CIN>(a, st);
+}
+
+template <int CIN>
+cudaError_t launch_wgrad_cin(int cout_pad, const WgradArgs &a, cudaStream_t st)
+{
+    switch (cout_pad) {
+    case 16: return launch_wgrad_t<CIN, 16>(a, st);
+    case 32: return launch_wgrad_t<CIN, 32>(a, st);
+    case 48: return launch_wgrad_t<CIN, 48>(a, st);
+    case 64: return launch_wgrad_t<CIN, 64>(a, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 // cin_pad, cout_pad: padded channel counts (multiples of 16)
-cudaError_t launch_wgrad(int cin_pad, int cout_pad, const __nv_bfloat16 *h, const __nv_bfloat16 *dzb, const float *dzf,
-                         int cin, int cout, int npix, int H, int W, float *dW, float *db, cudaStream_t st)
+cudaError_t launch_wgrad(int cin_pad, int cout_pad, const WgradArgs &a, cudaStream_t st)
 {
     switch (cin_pad) {
-    case 16: return launch_wgrad_cin<16>(cout_pad, h, dzb, dzf, cin, cout, npix, H, W, dW, db, st);
-    case 32: return launch_wgrad_cin<32>(cout_pad, h, dzb, dzf, cin, cout, npix, H, W, dW, db, st);
-    case 48: return launch_wgrad_cin<48>(cout_pad, h, dzb, dzf, cin, cout, npix, H, W, dW, db, st);
-    case 64: return launch_wgrad_cin<64>(cout_pad, h, dzb, dzf, cin, cout, npix, H, W, dW, db, st);
+    case 16: return launch_wgrad_cin<16>(cout_pad, a, st);
+    case 32: return launch_wgrad_cin<32>(cout_pad, a, st);
+    case 48: return launch_wgrad_cin<48>(cout_pad, a, st);
+    case 64: return launch_wgrad_cin<64>(cout_pad, a, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -599,6 +888,9 @@ struct ConvArgs {
     float *z;
     const float *zprev;
     int npix, H, W, mode, flip;
+    float *bpart = nullptr;  // mode 2: column sums of the FP32 result wanted (partial rows, BIAS_BLOCKS at most)
+    int *nb = nullptr;       // how many partial rows were written
+    bool keep_z = true;      // false: z serves the column sums only and need not be written
 };
 
 // Staged form for images whose width is a multiple of STG_TW: a CTA of 4
@@ -617,14 +909,6 @@ struct StagedConvGeom {
     static constexpr size_t w_elems = (size_t)NOUT * LDB;  // one tap
     static constexpr size_t smem_bytes = (in_elems + 2 * w_elems) * sizeof(__nv_bfloat16);
 };
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 template <int CIN, int NOUT>
 __global__ void __launch_bounds__(STG_THREADS)
@@ -903,12 +1187,13 @@ __device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float *v)
     }
 }
 
-template <int CIN, int NOUT>
+// BSUM: column sums of the FP32 results go to bpart (one row per CTA).
+template <int CIN, int NOUT, bool BSUM>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__restrict__ B,
                const float *__restrict__ bias, int nbias, __nv_bfloat16 *__restrict__ out_bf,
                float *__restrict__ z_f32, const float *__restrict__ zprev, int H, int W, int ntiles, int mode,
-               int flip)
+               int flip, float *__restrict__ bpart)
 {
     using G = TcGeom<CIN, NOUT>;
     constexpr int CH = G::CH, COLS = G::COLS;
@@ -976,6 +1261,14 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    // column sums of this thread's outputs over its tiles (bias gradient):
+    // FP32 sums of at most my_tiles values, taken from the registers that
+    // hold the result, so that the FP32 result need not be written and read
+    // again
+    fp2 bsum[COLS / 2];
+#pragma unroll
+    for (int c = 0; c < COLS / 2; c++) bsum[c] = bc2(0.0f);
+
     // epilogue of local tile k (accumulator k & 1): warp w reads TMEM lanes
     // 32 (w % 4) .. +31 (pixels) and columns COLS (w / 4) .. +COLS-1 (outputs).
     // Once tile k's MMAs are complete, the ring slot of its first input row
@@ -1011,6 +1304,10 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                 const fp2 d1 = mul2(fp2{v[4 * c + 2], v[4 * c + 3]}, gelu_grad2(fp2{g.z, g.w}));
                 v[4 * c] = d0.x; v[4 * c + 1] = d0.y; v[4 * c + 2] = d1.x; v[4 * c + 3] = d1.y;
             }
+        }
+        if constexpr (BSUM) {
+#pragma unroll
+            for (int c = 0; c < COLS / 2; c++) bsum[c] = add2(bsum[c], fp2{v[2 * c], v[2 * c + 1]});
         }
         if (z_f32) {
             float4 *zd = reinterpret_cast<float4 *>(z_f32 + o);
@@ -1107,10 +1404,36 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
     if (ok && my_tiles > 0 && tid < TC_EPI) epilogue(my_tiles - 1, [] {});
     tc_fence_before();
     __syncthreads();
+    if constexpr (BSUM) {
+        // lanes, then the four pixel quarters (the ring is free by now)
+        float *sb = reinterpret_cast<float *>(tc_smem + G::W_BYTES);  // [4][NOUT]
+        if (tid < TC_EPI) {
+#pragma unroll
+            for (int c = 0; c < COLS; c++) {
+                float x = c & 1 ? bsum[c / 2].y : bsum[c / 2].x;
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1) x += __shfl_down_sync(0xffffffffu, x, w);
+                if (lane == 0) sb[(warp & 3) * NOUT + COLS * (warp >> 2) + c] = x;
+            }
+        }
+        __syncthreads();
+        if (tid < NOUT)
+            bpart[(size_t)blockIdx.x * NOUT + tid] = (sb[tid] + sb[NOUT + tid]) + (sb[2 * NOUT + tid] + sb[3 * NOUT + tid]);
+    }
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(G::TMEM_COLS) : "memory");
     }
+}
+
+// Column sums of a convolution's FP32 result, where they are wanted.
+cudaError_t launch_colsum(const ConvArgs &a, int C, cudaStream_t st)
+{
+    if (a.bpart) {
+        colsum_kernel<<<BIAS_BLOCKS, 256, 0, st>>>(a.z, C, a.npix, a.bpart);
+        *a.nb = BIAS_BLOCKS;
+    }
+    return cudaGetLastError();
 }
 
 // Persistent grid: two CTAs per SM (the weights of a 64 x 64 layer take
@@ -1146,15 +1469,24 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st)
         if (a.W % TC_TW == 0 && a.npix % (a.H * a.W) == 0 && use_tc()) {
             static bool tc_ready = false;
             if (!tc_ready) {
-                const cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<CIN, NOUT>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+                cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<CIN, NOUT, false>,
+                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(conv_tc_kernel<CIN, NOUT, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
                 if (e != cudaSuccess) return e;
                 tc_ready = true;
             }
             const int ntiles = a.npix / TC_TW;
             const int blocks = ntiles < sms ? ntiles : sms;
-            conv_tc_kernel<CIN, NOUT><<<blocks, TC_THREADS, TC_SMEM, st>>>(a.in, a.B, a.bias, a.nbias, a.out, a.z,
-                                                                          a.zprev, a.H, a.W, ntiles, a.mode, a.flip);
+            float *z = a.keep_z ? a.z : nullptr;
+            if (a.bpart)
+                conv_tc_kernel<CIN, NOUT, true><<<blocks, TC_THREADS, TC_SMEM, st>>>(
+                    a.in, a.B, a.bias, a.nbias, a.out, z, a.zprev, a.H, a.W, ntiles, a.mode, a.flip, a.bpart);
+            else
+                conv_tc_kernel<CIN, NOUT, false><<<blocks, TC_THREADS, TC_SMEM, st>>>(
+                    a.in, a.B, a.bias, a.nbias, a.out, z, a.zprev, a.H, a.W, ntiles, a.mode, a.flip, nullptr);
+            if (a.bpart) *a.nb = blocks;
             return cudaGetLastError();
         }
     }
@@ -1169,13 +1501,13 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st)
         }
         conv_staged_kernel<CIN, NOUT><<<a.npix / STG_TW, STG_THREADS, S::smem_bytes, st>>>(
             a.in, a.B, a.bias, a.nbias, a.out, a.z, a.zprev, a.H, a.W, a.mode, a.flip);
-        return cudaGetLastError();
+        return launch_colsum(a, NOUT, st);
     }
     const int tiles = (a.npix + CONV_THREADS - 1) / CONV_THREADS;
     const int blocks = tiles < 2 * sms ? tiles : 2 * sms;
     conv_mma_kernel<CIN, NOUT><<<blocks, CONV_THREADS, G::smem_bytes, st>>>(a.in, a.B, a.bias, a.nbias, a.out, a.z,
                                                                           a.zprev, a.npix, a.H, a.W, a.mode, a.flip);
-    return cudaGetLastError();
+    return launch_colsum(a, NOUT, st);
 }
 
 template <int CIN>
@@ -1222,6 +1554,8 @@ struct hlbm_sur {
     float *y = nullptr;
     float *xin = nullptr;   // FP32 copy of the last forward input (residual path)
     double *loss = nullptr;
+    float *wpart = nullptr;  // partial weight gradients, one slice per pixel chunk
+    float *bpart = nullptr;  // partial bias gradients, BIAS_BLOCKS rows of MAXC
     int last_batch = 0;
     int64_t adam_t = 0;
 };
@@ -1236,6 +1570,7 @@ void hlbm_sur_destroy(hlbm_sur *s)
     for (int l = 0; l < MAX_LAYERS; l++) { cudaFree(s->Wb[l]); cudaFree(s->Wd[l]); cudaFree(s->z[l]); }
     for (int l = 0; l <= MAX_LAYERS; l++) cudaFree(s->act[l]);
     cudaFree(s->gbuf[0]); cudaFree(s->gbuf[1]); cudaFree(s->dz); cudaFree(s->dz2); cudaFree(s->y); cudaFree(s->xin); cudaFree(s->loss);
+    cudaFree(s->wpart); cudaFree(s->bpart);
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     delete s;
 }
@@ -1278,6 +1613,13 @@ int hlbm_sur_create(int nlayer, const int *widths, int H, int W, int batch_max, 
               cudaMalloc(&s->dz, npix * MAXC * 4) == cudaSuccess && cudaMalloc(&s->dz2, npix * MAXC * 4) == cudaSuccess &&
               cudaMalloc(&s->gbuf[0], npix * MAXC * 2) == cudaSuccess &&
               cudaMalloc(&s->gbuf[1], npix * MAXC * 2) == cudaSuccess;
+    size_t wpart = 0;
+    for (int l = 0; l < nlayer; l++) {
+        const size_t n = (npix + WG_CHUNK - 1) / WG_CHUNK * 9 * s->cpad_in[l] * s->cpad_out[l];
+        wpart = n > wpart ? n : wpart;
+    }
+    ok = ok && cudaMalloc(&s->wpart, wpart * 4) == cudaSuccess &&
+         cudaMalloc(&s->bpart, (size_t)BIAS_BLOCKS * MAXC * 4) == cudaSuccess;
     for (int l = 0; l < nlayer && ok; l++) {
         ok = cudaMalloc(&s->Wb[l], (size_t)9 * s->cpad_out[l] * s->cpad_in[l] * 2) == cudaSuccess &&
              cudaMalloc(&s->Wd[l], (size_t)9 * s->cpad_out[l] * s->cpad_in[l] * 2) == cudaSuccess &&
@@ -1409,12 +1751,18 @@ static int sur_backward(hlbm_sur *s, const float *target, const float *dy, int a
     // BF16 copy of the top gradient for the tensor-core input-gradient pass
     to_bf16_kernel<<<1024, 256, 0, s->stream>>>(dzf[cur], (long long)npix * s->cpad_out[L - 1], s->gbuf[0]);
     if (cudaGetLastError() != cudaSuccess) return HLBM_ERR_CUDA;
-    int gb = 0;
+    // partial sums of the bias gradient of layer l: of the top layer from the
+    // FP32 gradient itself, of the others from the pass that computes dz_l
+    int gb = 0, nb = BIAS_BLOCKS;
+    colsum_kernel<<<BIAS_BLOCKS, 256, 0, s->stream>>>(dzf[cur], s->cpad_out[L - 1], npix, s->bpart);
+    if (cudaGetLastError() != cudaSuccess) return HLBM_ERR_CUDA;
     for (int l = L - 1; l >= 0; l--) {
         // weight gradient on the tensor cores from the BF16 copy of dz_l
-        if (launch_wgrad(s->cpad_in[l], s->cpad_out[l], s->act[l], s->gbuf[gb], dzf[cur], s->width[l], s->width[l + 1],
-                         npix, s->H, s->W, s->g + s->woff[l], s->g + s->boff[l], s->stream) != cudaSuccess)
-            return HLBM_ERR_CUDA;
+        const WgradArgs wa{s->act[l], s->gbuf[gb], s->width[l], s->width[l + 1], npix, s->H, s->W,
+                           s->g + s->woff[l], s->wpart};
+        if (launch_wgrad(s->cpad_in[l], s->cpad_out[l], wa, s->stream) != cudaSuccess) return HLBM_ERR_CUDA;
+        bias_reduce_kernel<<<s->width[l + 1], 32, 0, s->stream>>>(s->bpart, nb, s->cpad_out[l], s->g + s->boff[l]);
+        if (cudaGetLastError() != cudaSuccess) return HLBM_ERR_CUDA;
         if (l == 0) {
             if (dx) {
                 // the network's part of dL/dx: W_0^T * dz_0, the transposed
@@ -1428,10 +1776,14 @@ static int sur_backward(hlbm_sur *s, const float *target, const float *dy, int a
             break;
         }
         // dz_{l-1} = (W_l^T * dz_l) . GELU'(z_{l-1}): the transposed
-        // convolution on the tensor cores (dz read at p - offset(tap)),
-        // GELU' in the epilogue, FP32 and BF16 results
-        const ConvArgs a{s->gbuf[gb], s->Wd[l], nullptr, 0, s->gbuf[gb ^ 1], dzf[cur ^ 1], s->z[l - 1], npix, s->H,
-                         s->W, 2, 1};
+        // convolution on the tensor cores (dz read at p - offset(tap)), GELU'
+        // in the epilogue; the BF16 result feeds the next layer, the FP32
+        // result only its bias gradient
+        ConvArgs a{s->gbuf[gb], s->Wd[l], nullptr, 0, s->gbuf[gb ^ 1], dzf[cur ^ 1], s->z[l - 1], npix, s->H,
+                   s->W, 2, 1};
+        a.bpart = s->bpart;
+        a.nb = &nb;
+        a.keep_z = false;
         if (launch_conv(s->cpad_out[l], s->cpad_in[l], a, s->stream) != cudaSuccess) return HLBM_ERR_CUDA;
         cur ^= 1;
         gb ^= 1;
