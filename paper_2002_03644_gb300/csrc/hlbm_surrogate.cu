@@ -1024,16 +1024,22 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 //   - the nine taps' weights stay in shared memory for the whole launch;
 //   - each 128-pixel row segment is one M = 128 tile; a CTA walks down a
 //     contiguous run of tiles of one column segment, so consecutive tiles
-//     share two of their three input rows.  The rows live in a ring of five
-//     shared-memory slots: the current tile's three, the next tile's new
-//     row, and the row after it, copied two tiles ahead (a run that crosses
-//     an image refills the ring);
-//   - one thread issues a tile's 9 CIN / 16 MMAs (M = 128, N = NOUT, K = 16,
-//     BF16 operands) into one of two TMEM accumulators of NOUT FP32 columns,
-//     with tcgen05.commit signalling an mbarrier when they are done;
-//   - while the MMAs of tile k run, all warps read tile k-1's accumulator
-//     (tcgen05.ld), apply bias / GELU and store.
-//   - warps 0-15 copy rows and run the epilogue; warp 16 only issues MMAs.
+//     share two of their three input rows, which live in a ring of row slots;
+//   - the roles run apart and meet at mbarriers only: warp 17 copies rows
+//     ahead (cp.async) as slots come free; one thread of warp 16 issues a
+//     tile's 9 CIN / 16 MMAs (M = 128, N = NOUT, K = 16, BF16 operands) into
+//     one of two TMEM accumulators of NOUT FP32 columns, with tcgen05.commit
+//     signalling the accumulator and the freed row slots; warps 0-7 and 8-15
+//     take the even and the odd tiles' accumulators (tcgen05.ld), give the
+//     accumulator back as soon as it is in registers, apply bias / GELU and
+//     store.
+// What bounds it: a 64 -> 64 tile's 36 MMAs take 48 cycles each (each reads
+// 6 KB of operands from shared memory at 128 B per clock; N = 128 would be
+// the first shape that runs at the tensor core's own rate), 1740 cycles, and
+// its GELUs 1024 cycles of the MUFU (two per value).  With all warps in one
+// loop behind a barrier per tile, the copy, the TMEM read, the GELU and the
+// stores of a tile stood one after another and a tile took 4500 cycles: 133
+// us per 64 -> 64 layer of 16 x 256^2, against @NEW@ with the roles apart.
 // Operands are K-major.  With 64 channels a pixel (or a weight row) is one
 // 128-byte row of the 128-byte swizzle layout, so a tap's pixel shift moves
 // the operand by whole aligned rows.  With 16 channels they use the layout
@@ -1041,11 +1047,10 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 // 8-row groups SBO = 128 bytes apart (consecutive pixels are consecutive
 // 16-byte rows and a pixel shift is a 16-byte offset of the start
 // address), the two 8-channel halves of a K-slice LBO bytes apart.
-constexpr int TC_THREADS = 544, TC_TW = 128, TC_RW = TC_TW + 2;
-constexpr int TC_EPI = 512;        // warps 0-15: copies and epilogue; warp 16 issues the MMAs
-constexpr int TC_MMA_TID = 512;
+constexpr int TC_THREADS = 576, TC_TW = 128, TC_RW = TC_TW + 2;
+constexpr int TC_MMA_WARP = 16, TC_COPY_WARP = 17;
 constexpr uint32_t TC_IN_LBO = TC_RW * 16;               // 2080: channel-chunk stride of a staged row
-// Dynamic shared memory requested: the operands need at most 173.6 KB (64 ->
+// Dynamic shared memory requested: the operands need at most 178.7 KB (64 ->
 // 64); the rest is slack so that every address a descriptor can form stays
 // inside the block.
 constexpr uint32_t TC_SMEM = 220 * 1024;
@@ -1065,17 +1070,21 @@ struct TcGeom {
     static constexpr uint32_t W_BYTES = 9 * W_TAP;
     static constexpr uint32_t IN_ROW = SW ? (TC_RW * 128 + 1023) / 1024 * 1024  // [column][128 B]
                                           : CH * TC_IN_LBO;                       // [k / 8][column][8]
-    static constexpr int SLOTS = 5;                              // row ring
-    static constexpr uint32_t BAR_OFF = W_BYTES + SLOTS * IN_ROW;  // two mbarriers, then the TMEM address
-    static constexpr uint32_t BIAS_OFF = BAR_OFF + 32;           // NOUT FP32 bias values
+    static constexpr int SLOTS = 6;                              // row ring
+    static constexpr uint32_t BAR_OFF = W_BYTES + SLOTS * IN_ROW;  // mbarriers (BAR_*), then the TMEM address
+    static constexpr int BAR_FULL = 0, BAR_FREE = SLOTS;         // row slots: copied / read by the MMAs
+    static constexpr int BAR_ACC = 2 * SLOTS, BAR_OUT = 2 * SLOTS + 2;  // accumulators: computed / read
+    static constexpr int NBAR = 2 * SLOTS + 4;
+    static constexpr uint32_t BIAS_OFF = BAR_OFF + 8 * NBAR + 16;  // NOUT FP32 bias values
     static constexpr uint32_t TMEM_COLS = 2 * NOUT < 32 ? 32 : 2 * NOUT;  // two accumulators (allocation >= 32)
-    static constexpr int COLS = NOUT / 4;                        // accumulator columns per warp in the epilogue
+    static constexpr int COLS = NOUT / 2;                        // accumulator columns per epilogue warp
+    static constexpr int HC = COLS < 16 ? COLS : 16;             // columns taken at once
     // Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1),
     // BF16 A and B (bits 7-9, 10-12 = 1), both K-major, N >> 3 at bit 17,
     // M >> 4 at bit 24.
     static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NOUT >> 3) << 17) |
                                       ((uint32_t)(TC_TW >> 4) << 24);
-    static_assert(BIAS_OFF + 4 * NOUT <= TC_SMEM, "shared memory");
+    static_assert(BIAS_OFF % 16 == 0 && BIAS_OFF + 9 * 4 * NOUT <= TC_SMEM, "shared memory");
     static_assert(!SW || (W_TAP % 1024 == 0 && W_BYTES % 1024 == 0 && IN_ROW % 1024 == 0), "swizzle atoms");
     static_assert(NOUT % 16 == 0 && CIN % 16 == 0, "shapes");
 };
@@ -1158,33 +1167,39 @@ __device__ __forceinline__ void tmem_ld<16>(uint32_t taddr, float *v)
     for (int k = 0; k < 16; k++) v[k] = __uint_as_float(r[k]);
 }
 template <>
-__device__ __forceinline__ void tmem_ld<4>(uint32_t taddr, float *v)
+__device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, float *v)
 {
-    uint32_t r[4];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int k = 0; k < 4; k++) v[k] = __uint_as_float(r[k]);
+    for (int k = 0; k < 8; k++) v[k] = __uint_as_float(r[k]);
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// 16 bytes: COLS / ... BF16 values of out (COLS = 4: 8 bytes)
-template <int COLS>
+// N (a multiple of 8) BF16 values in 16-byte stores
+template <int N>
 __device__ __forceinline__ void store_bf16(__nv_bfloat16 *dst, const float *v)
 {
-    if constexpr (COLS == 4) {
-        *reinterpret_cast<uint2 *>(dst) = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
-    } else {
-        uint4 *d = reinterpret_cast<uint4 *>(dst);
+    uint4 *d = reinterpret_cast<uint4 *>(dst);
 #pragma unroll
-        for (int c = 0; c < COLS / 8; c++)
-            d[c] = make_uint4(pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
-                              pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
-    }
+    for (int c = 0; c < N / 8; c++)
+        d[c] = make_uint4(pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
+                          pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
+}
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 // BSUM: column sums of the FP32 results go to bpart (one row per CTA).
@@ -1196,12 +1211,12 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                int flip, float *__restrict__ bpart)
 {
     using G = TcGeom<CIN, NOUT>;
-    constexpr int CH = G::CH, COLS = G::COLS;
+    constexpr int CH = G::CH, COLS = G::COLS, HC = G::HC, SLOTS = G::SLOTS;
     extern __shared__ __align__(1024) unsigned char tc_smem[];
     const uint32_t sbase = smem_addr(tc_smem);
     const uint32_t w_s = sbase, ring_s = sbase + G::W_BYTES;
     auto bar = [&](int b) { return sbase + G::BAR_OFF + 8 * b; };
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tc_smem + G::BAR_OFF + 16);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tc_smem + G::BAR_OFF + 8 * G::NBAR);
     float *bias_s = reinterpret_cast<float *>(tc_smem + G::BIAS_OFF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nseg = W / TC_TW;
@@ -1220,8 +1235,11 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar(0)) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar(1)) : "memory");
+        // one arrival each: the copying warp's, a commit's, or (an
+        // accumulator read) one per warp of its group
+        for (int b = 0; b < G::BAR_OUT; b++) mbar_init(bar(b), 1);
+        mbar_init(bar(G::BAR_OUT), 8);
+        mbar_init(bar(G::BAR_OUT + 1), 8);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // weights of all taps: B[tap][n][k] -> [tap][k / 8][n][8]
@@ -1230,195 +1248,229 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
         const uint32_t off = G::SW ? nrow * 128 + ((kc ^ (nrow & 7)) << 4) : kc * G::W_LBO + nrow * 16;
         cp_async16(tc_smem + tap * G::W_TAP + off, B + ((size_t)tap * NOUT + nrow) * CIN + kc * 8);
     }
-    // Tiles are numbered column segment first: T = seg R + r, r = n H + i;
-    // this CTA takes T in [t0, t0 + my_tiles).  Tile T + 1 shares two input
-    // rows with T unless T is an image's last row (or the segment's).
-    const int t0 = (int)(((long long)blockIdx.x * ntiles) / gridDim.x);
-    const int my_tiles = (int)(((long long)(blockIdx.x + 1) * ntiles) / gridDim.x) - t0;
-    auto successor = [&](int T) { return (T % H) != H - 1; };
-    // input row i - 1 + d (wrapped in the image) of tile T, columns j0-1 ..
-    // j0+128 -> ring slot [k / 8][column][8]: thread t copies channel chunk
-    // t % CH of columns t / CH + (512 / CH) m
-    const int s_kc = tid % CH, s_px = tid / CH;
-    auto load_row = [&](int T, int d, int slot) {
-        if (tid >= TC_EPI) return;
-        const int seg = T / R, r = T - seg * R;
-        const int n = r / H, i = r - n * H, j0 = seg * TC_TW;
-        const __nv_bfloat16 *src = in + ((size_t)n * H + wrap(i - 1 + d, H)) * W * CIN + s_kc * 8;
-        unsigned char *dst = tc_smem + G::W_BYTES + slot * G::IN_ROW;
-#pragma unroll
-        for (int m = 0; m < (TC_RW * CH + TC_EPI - 1) / TC_EPI; m++) {
-            const int px = s_px + (TC_EPI / CH) * m;
-            const uint32_t off = G::SW ? px * 128 + ((s_kc ^ (px & 7)) << 4) : s_kc * TC_IN_LBO + px * 16;
-            if (px < TC_RW) cp_async16(dst + off, src + (size_t)wrap(j0 + px - 1, W) * CIN);
-        }
-    };
     cp_async_commit();
-    cp_async_wait0();  // the weights
+    cp_async_wait0();
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // column sums of this thread's outputs over its tiles (bias gradient):
-    // FP32 sums of at most my_tiles values, taken from the registers that
-    // hold the result, so that the FP32 result need not be written and read
-    // again
-    fp2 bsum[COLS / 2];
-#pragma unroll
-    for (int c = 0; c < COLS / 2; c++) bsum[c] = bc2(0.0f);
+    // Tiles are numbered column segment first: T = seg R + r, r = n H + i;
+    // this CTA takes T in [t0, t0 + my_tiles).  Tile T + 1 shares two input
+    // rows with T unless T is an image's last row (or the segment's).  The
+    // rows a CTA copies form one stream: q counts them, row q sits in slot
+    // q % SLOTS, and a tile's rows are q0, q0 + 1, q0 + 2 with q0 one further
+    // than its predecessor's (three further when it starts a new run).
+    const int t0 = (int)(((long long)blockIdx.x * ntiles) / gridDim.x);
+    const int my_tiles = (int)(((long long)(blockIdx.x + 1) * ntiles) / gridDim.x) - t0;
 
-    // epilogue of local tile k (accumulator k & 1): warp w reads TMEM lanes
-    // 32 (w % 4) .. +31 (pixels) and columns COLS (w / 4) .. +COLS-1 (outputs).
-    // Once tile k's MMAs are complete, the ring slot of its first input row
-    // is free: then() copies a later tile's row into it right away, so that
-    // the copy overlaps the epilogue math.
-    auto epilogue = [&](int k, auto then) -> bool {
-        const int T = t0 + k;
-        // the warp-wide TMEM load below needs the whole warp: agree on the outcome
-        if (!__all_sync(0xffffffffu, mbar_wait(bar(k & 1), (k >> 1) & 1))) return false;
-        then();
-        tc_fence_after();
-        const int q = warp & 3, h = warp >> 2;
-        float v[COLS];
-        tmem_ld<COLS>(tmem + ((uint32_t)(32 * q) << 16) + (k & 1) * NOUT + COLS * h, v);
-        const int seg = T / R, r = T - seg * R;
-        const size_t p = (size_t)r * W + seg * TC_TW + 32 * q + lane;
-        const size_t o = p * NOUT + COLS * h;  // this thread's COLS outputs
-        // pairs of adjacent outputs in packed FP32
-        const float2 *bs = reinterpret_cast<const float2 *>(bias_s + COLS * h);
-#pragma unroll
-        for (int c = 0; c < COLS / 2; c++) {
-            const float2 b2 = bs[c];
-            const fp2 z = add2(fp2{v[2 * c], v[2 * c + 1]}, fp2{b2.x, b2.y});
-            v[2 * c] = z.x;
-            v[2 * c + 1] = z.y;
+    if (warp == TC_COPY_WARP) {
+        // ---- rows: lane l copies channel chunk l % CH of columns l / CH + (32 / CH) m
+        const int kc = lane % CH, px0 = lane / CH;
+        constexpr int STEP = 32 / CH;
+        auto load_row = [&](int seg, int n, int i, int d, int slot) {  // input row i - 1 + d, columns j0 - 1 .. j0 + 128
+            const int j0 = seg * TC_TW;
+            const __nv_bfloat16 *src = in + ((size_t)n * H + wrap(i - 1 + d, H)) * W * CIN + kc * 8;
+            unsigned char *dst = tc_smem + G::W_BYTES + slot * G::IN_ROW;
+#pragma unroll 8
+            for (int px = px0; px < TC_RW; px += STEP) {
+                const uint32_t off = G::SW ? px * 128 + ((kc ^ (px & 7)) << 4) : kc * TC_IN_LBO + px * 16;
+                int j = j0 + px - 1;
+                j = j < 0 ? j + W : (j >= W ? j - W : j);
+                cp_async16(dst + off, src + (size_t)j * CIN);
+            }
+        };
+        // Row q is announced once its copies are complete; two more rows may
+        // be in flight by then.  Before the warp waits for a slot it
+        // announces everything it has copied: the MMAs that free the slot may
+        // need those rows.
+        int q = 0, told = 0;
+        auto tell = [&](int upto) {
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0)
+                for (int e = told; e < upto; e++) mbar_arrive(bar(G::BAR_FULL + e % SLOTS));
+            told = upto;
+        };
+        bool ok = true;
+        int seg = t0 / R, r = t0 - seg * R, n = r / H, i = r - n * H;
+        for (int k = 0; k < my_tiles && ok; k++) {
+            for (int d = (k == 0 || i == 0) ? 0 : 2; d < 3 && ok; d++) {
+                const int slot = q % SLOTS;
+                if (q >= SLOTS) {
+                    const uint32_t parity = (q / SLOTS - 1) & 1;
+                    if (!__all_sync(0xffffffffu, mbar_try_wait(bar(G::BAR_FREE + slot), parity))) {
+                        cp_async_wait0();
+                        tell(q);
+                        ok = __all_sync(0xffffffffu, mbar_wait(bar(G::BAR_FREE + slot), parity));
+                        if (!ok) break;
+                    }
+                }
+                load_row(seg, n, i, d, slot);
+                cp_async_commit();
+                q++;
+                if (q - told > 2) {
+                    asm volatile("cp.async.wait_group 2;" ::: "memory");
+                    tell(q - 2);
+                }
+            }
+            if (++i == H) {
+                i = 0;
+                if (++n * H == R) { n = 0; seg++; }
+            }
         }
-        if (mode == 2 && zprev) {
-            const float4 *zp = reinterpret_cast<const float4 *>(zprev + o);
+        cp_async_wait0();
+        tell(q);
+    } else if (warp == TC_MMA_WARP) {
+        if (lane == 0) {
+            // ---- the MMAs of a tile whose input rows i-1, i, i+1 sit in slots
+            // (q0 + 0, 1, 2) % SLOTS: a K-slice of tap (dp, dq) starts at row
+            // slot (q0 + 1 + dp), column 1 + dq; descriptors differ from the
+            // slot's only in the start-address field (16-byte units).
+            const uint64_t bdesc0 = G::SW ? umma_desc_sw(w_s) : umma_desc(w_s, G::W_LBO, 128);
+            auto issue = [&](uint32_t d, int q0, bool flipped) {
+                uint64_t rowdesc[3];
 #pragma unroll
-            for (int c = 0; c < COLS / 4; c++) {
-                const float4 g = zp[c];
-                const fp2 d0 = mul2(fp2{v[4 * c], v[4 * c + 1]}, gelu_grad2(fp2{g.x, g.y}));
-                const fp2 d1 = mul2(fp2{v[4 * c + 2], v[4 * c + 3]}, gelu_grad2(fp2{g.z, g.w}));
-                v[4 * c] = d0.x; v[4 * c + 1] = d0.y; v[4 * c + 2] = d1.x; v[4 * c + 3] = d1.y;
+                for (int e = 0; e < 3; e++) {
+                    const uint32_t a = ring_s + ((q0 + e) % SLOTS) * G::IN_ROW;
+                    rowdesc[e] = G::SW ? umma_desc_sw(a) : umma_desc(a, TC_IN_LBO, 128);
+                }
+#pragma unroll
+                for (int tap = 0; tap < 9; tap++) {
+                    const int dp = flipped ? 1 - tap / 3 : tap / 3 - 1, dq = flipped ? 1 - tap % 3 : tap % 3 - 1;
+#pragma unroll
+                    for (int ks = 0; ks < CIN / 16; ks++) {
+                        // start-address offsets: the pixel shift (whole 128-byte rows
+                        // when swizzled) and the K-slice (32 bytes within the row)
+                        const uint32_t ao = G::SW ? ((1 + dq) * 128 + 32 * ks) >> 4 : ((1 + dq) * 16 + 2 * ks * TC_IN_LBO) >> 4;
+                        const uint32_t bo = G::SW ? (tap * G::W_TAP + 32 * ks) >> 4 : (tap * G::W_TAP + 2 * ks * G::W_LBO) >> 4;
+                        umma_f16(d, rowdesc[1 + dp] + ao, bdesc0 + bo, G::IDESC, (tap | ks) != 0);
+                    }
+                }
+            };
+            bool ok = true;
+            int q0 = 0, q = 0;  // the tile's first row; rows known to be copied
+            int i = t0 % H;
+            for (int k = 0; k < my_tiles && ok; k++) {
+                const bool last = k + 1 == my_tiles || i == H - 1;  // of its run
+                if (k >= 2) ok = mbar_wait(bar(G::BAR_OUT + (k & 1)), ((k >> 1) - 1) & 1);
+                for (; ok && q < q0 + 3; q++) ok = mbar_wait(bar(G::BAR_FULL + q % SLOTS), (q / SLOTS) & 1);
+                if (!ok) break;
+                tc_fence_after();
+                if (flip) issue(tmem + (k & 1) * NOUT, q0, true);
+                else issue(tmem + (k & 1) * NOUT, q0, false);
+                umma_commit(bar(G::BAR_ACC + (k & 1)));
+                for (int e = 0; e < (last ? 3 : 1); e++) umma_commit(bar(G::BAR_FREE + (q0 + e) % SLOTS));
+                if (k + 1 == my_tiles)  // no arrival may be outstanding when the CTA ends
+                    for (int e = 0; e < 3; e++) mbar_wait(bar(G::BAR_FREE + (q0 + e) % SLOTS), ((q0 + e) / SLOTS) & 1);
+                q0 += last ? 3 : 1;
+                i = i == H - 1 ? 0 : i + 1;
+            }
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue: warp w takes TMEM lanes 32 (w % 4) .. +31 (pixels) and
+        // columns COLS ((w / 4) % 2) .. +COLS-1 (outputs) of the tiles of its group
+        const int q = warp & 3, h = (warp >> 2) & 1, grp = warp >> 3;
+        // column sums of this thread's outputs over its tiles (bias gradient):
+        // FP32 sums of at most my_tiles values, taken from the registers that
+        // hold the result, so that the FP32 result need not be written and read
+        // again
+        fp2 bsum[BSUM ? COLS / 2 : 1];
+#pragma unroll
+        for (int c = 0; c < (BSUM ? COLS / 2 : 1); c++) bsum[c] = bc2(0.0f);
+        int seg = (t0 + grp) / R, r = (t0 + grp) - seg * R;
+        for (int k = grp; k < my_tiles; k += 2) {
+            const size_t p = (size_t)r * W + seg * TC_TW + 32 * q + lane;
+            const size_t o = p * NOUT + COLS * h;  // this thread's COLS outputs
+            r += 2;
+            while (r >= R) { r -= R; seg++; }
+            // the pre-activations of the backward pass do not depend on the
+            // MMAs: the first ones are under way while those run
+            float4 zp[HC / 4];
+            if (mode == 2 && zprev) {
+#pragma unroll
+                for (int c = 0; c < HC / 4; c++) zp[c] = reinterpret_cast<const float4 *>(zprev + o)[c];
+            }
+            // the warp-wide TMEM load below needs the whole warp: agree on the outcome
+            if (!__all_sync(0xffffffffu, mbar_wait(bar(G::BAR_ACC + grp), (k >> 1) & 1))) break;
+            tc_fence_after();
+#pragma unroll
+            for (int c0 = 0; c0 < COLS; c0 += HC) {
+                float v[HC];
+                tmem_ld<HC>(tmem + ((uint32_t)(32 * q) << 16) + grp * NOUT + COLS * h + c0, v);
+                if (c0 + HC == COLS) {
+                    // all of this warp's part is in registers: the accumulator may be overwritten
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(G::BAR_OUT + grp));
+                }
+                // pairs of adjacent outputs in packed FP32
+                const float2 *bs = reinterpret_cast<const float2 *>(bias_s + COLS * h + c0);
+#pragma unroll
+                for (int c = 0; c < HC / 2; c++) {
+                    const float2 b2 = bs[c];
+                    const fp2 z = add2(fp2{v[2 * c], v[2 * c + 1]}, fp2{b2.x, b2.y});
+                    v[2 * c] = z.x;
+                    v[2 * c + 1] = z.y;
+                }
+                if (mode == 2 && zprev) {
+                    if (c0 > 0) {
+#pragma unroll
+                        for (int c = 0; c < HC / 4; c++) zp[c] = reinterpret_cast<const float4 *>(zprev + o + c0)[c];
+                    }
+#pragma unroll
+                    for (int c = 0; c < HC / 4; c++) {
+                        const float4 g = zp[c];
+                        const fp2 d0 = mul2(fp2{v[4 * c], v[4 * c + 1]}, gelu_grad2(fp2{g.x, g.y}));
+                        const fp2 d1 = mul2(fp2{v[4 * c + 2], v[4 * c + 3]}, gelu_grad2(fp2{g.z, g.w}));
+                        v[4 * c] = d0.x; v[4 * c + 1] = d0.y; v[4 * c + 2] = d1.x; v[4 * c + 3] = d1.y;
+                    }
+                }
+                if constexpr (BSUM) {
+#pragma unroll
+                    for (int c = 0; c < HC / 2; c++)
+                        bsum[c0 / 2 + c] = add2(bsum[c0 / 2 + c], fp2{v[2 * c], v[2 * c + 1]});
+                }
+                if (z_f32) {
+                    float4 *zd = reinterpret_cast<float4 *>(z_f32 + o + c0);
+#pragma unroll
+                    for (int c = 0; c < HC / 4; c++) zd[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                }
+                if (mode == 1) {
+#pragma unroll
+                    for (int c = 0; c < HC / 2; c++) {
+                        const fp2 gv = gelu2(fp2{v[2 * c], v[2 * c + 1]});
+                        v[2 * c] = gv.x;
+                        v[2 * c + 1] = gv.y;
+                    }
+                }
+                store_bf16<HC>(out_bf + o + c0, v);
             }
         }
         if constexpr (BSUM) {
-#pragma unroll
-            for (int c = 0; c < COLS / 2; c++) bsum[c] = add2(bsum[c], fp2{v[2 * c], v[2 * c + 1]});
-        }
-        if (z_f32) {
-            float4 *zd = reinterpret_cast<float4 *>(z_f32 + o);
-#pragma unroll
-            for (int c = 0; c < COLS / 4; c++) zd[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-        }
-        if (mode == 1) {
-#pragma unroll
-            for (int c = 0; c < COLS / 2; c++) {
-                const fp2 gv = gelu2(fp2{v[2 * c], v[2 * c + 1]});
-                v[2 * c] = gv.x;
-                v[2 * c + 1] = gv.y;
-            }
-        }
-        store_bf16<COLS>(out_bf + o, v);
-        return true;
-    };
-
-    // The MMAs of a tile whose input rows i-1, i, i+1 sit in ring slots
-    // (base + 0, 1, 2) % 5: a K-slice of tap (dp, dq) starts at row slot
-    // (base + 1 + dp), column 1 + dq; descriptors differ from the slot's
-    // only in the start-address field (16-byte units).
-    const uint64_t bdesc0 = G::SW ? umma_desc_sw(w_s) : umma_desc(w_s, G::W_LBO, 128);
-    auto issue = [&](int b, int base, bool flipped) {
-        const uint32_t d = tmem + b * NOUT;
-        uint64_t rowdesc[3];
-#pragma unroll
-        for (int e = 0; e < 3; e++) {
-            const uint32_t a = ring_s + ((base + e) % G::SLOTS) * G::IN_ROW;
-            rowdesc[e] = G::SW ? umma_desc_sw(a) : umma_desc(a, TC_IN_LBO, 128);
-        }
-#pragma unroll
-        for (int tap = 0; tap < 9; tap++) {
-            const int dp = flipped ? 1 - tap / 3 : tap / 3 - 1, dq = flipped ? 1 - tap % 3 : tap % 3 - 1;
-#pragma unroll
-            for (int ks = 0; ks < CIN / 16; ks++) {
-                // start-address offsets: the pixel shift (whole 128-byte rows
-                // when swizzled) and the K-slice (32 bytes within the row)
-                const uint32_t ao = G::SW ? ((1 + dq) * 128 + 32 * ks) >> 4 : ((1 + dq) * 16 + 2 * ks * TC_IN_LBO) >> 4;
-                const uint32_t bo = G::SW ? (tap * G::W_TAP + 32 * ks) >> 4 : (tap * G::W_TAP + 2 * ks * G::W_LBO) >> 4;
-                umma_f16(d, rowdesc[1 + dp] + ao, bdesc0 + bo, G::IDESC, (tap | ks) != 0);
-            }
-        }
-        umma_commit(bar(b));
-    };
-
-    bool ok = true;
-    int j0 = 0;  // local index of the tile that started the current run
-    for (int k = 0; k < my_tiles && ok; k++) {
-        const int T = t0 + k;
-        if (k == 0 || !successor(T - 1)) {
-            // a new run: wait until the ring is free (the previous tile's
-            // MMAs are done), then copy this tile's three rows and the next
-            // tile's new row
-            if (k > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar((k - 1) & 1), ((k - 1) >> 1) & 1));
-            ok = __syncthreads_and(ok);
-            if (!ok) break;
-            j0 = k;
-            for (int d = 0; d < 3; d++) load_row(T, d, d);
-            if (k + 1 < my_tiles && successor(T)) load_row(T + 1, 2, 3);
-            cp_async_commit();
-            cp_async_wait0();
-            fence_async_smem();
-            tc_fence_before();
-            __syncthreads();
-        }
-        const int base = k - j0;
-        if (tid == TC_MMA_TID) {
-            // the MMAs of tile k into accumulator k & 1
-            tc_fence_after();
-            if (flip) issue(k & 1, base, true);
-            else issue(k & 1, base, false);
-        }
-        // tile k+2's new row, into the slot tile k-1's MMAs release
-        auto prefetch = [&]() {
-            if (k + 2 < my_tiles && successor(T) && successor(T + 1)) load_row(T + 2, 2, (base + 4) % G::SLOTS);
-        };
-        // tile k-1's results while tile k's MMAs run (warps 0-15)
-        if (tid < TC_EPI) {
-            if (k > 0) {
-                if (!epilogue(k - 1, prefetch)) ok = false;
-            } else {
-                prefetch();
-            }
-        }
-        cp_async_commit();
-        // tile k+1's new row (copied one iteration earlier) has arrived; the
-        // row of tile k+2 may still be in flight
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        fence_async_smem();
-        tc_fence_before();
-        ok = __syncthreads_and(ok);
-    }
-    if (ok && my_tiles > 0 && tid < TC_EPI) epilogue(my_tiles - 1, [] {});
-    tc_fence_before();
-    __syncthreads();
-    if constexpr (BSUM) {
-        // lanes, then the four pixel quarters (the ring is free by now)
-        float *sb = reinterpret_cast<float *>(tc_smem + G::W_BYTES);  // [4][NOUT]
-        if (tid < TC_EPI) {
+            // the sum over the lanes of a warp
+            float *sb = bias_s + NOUT;  // [8 = (group, pixel quarter)][NOUT]
 #pragma unroll
             for (int c = 0; c < COLS; c++) {
                 float x = c & 1 ? bsum[c / 2].y : bsum[c / 2].x;
 #pragma unroll
                 for (int w = 16; w > 0; w >>= 1) x += __shfl_down_sync(0xffffffffu, x, w);
-                if (lane == 0) sb[(warp & 3) * NOUT + COLS * (warp >> 2) + c] = x;
+                if (lane == 0) sb[(grp * 4 + q) * NOUT + COLS * h + c] = x;
             }
         }
-        __syncthreads();
-        if (tid < NOUT)
-            bpart[(size_t)blockIdx.x * NOUT + tid] = (sb[tid] + sb[NOUT + tid]) + (sb[2 * NOUT + tid] + sb[3 * NOUT + tid]);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if constexpr (BSUM) {
+        if (tid < NOUT) {
+            const float *sb = bias_s + NOUT;
+            float x = 0.0f;
+#pragma unroll
+            for (int e = 0; e < 8; e++) x += sb[e * NOUT + tid];
+            bpart[(size_t)blockIdx.x * NOUT + tid] = x;
+        }
     }
     if (warp == 0) {
         tc_fence_after();
