@@ -18,6 +18,7 @@
 // h[pixel + offset(tap), ci], a GEMM over pixels on the tensor cores
 // (BF16 operands, FP32 accumulators) whose partial sums are added up in a
 // fixed order.
+#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -891,6 +892,8 @@ struct ConvArgs {
     float *bpart = nullptr;  // mode 2: column sums of the FP32 result wanted (partial rows, BIAS_BLOCKS at most)
     int *nb = nullptr;       // how many partial rows were written
     bool keep_z = true;      // false: z serves the column sums only and need not be written
+    const CUtensorMap *ld = nullptr, *st = nullptr;  // of in / out where they have 64 channels (tcgen05 kernel)
+    bool zblk = false;       // pre-activations in blocks of 128 pixels (tcgen05 kernel): z of mode 1, zprev
 };
 
 // Staged form for images whose width is a multiple of STG_TW: a CTA of 4
@@ -1026,13 +1029,20 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 //     contiguous run of tiles of one column segment, so consecutive tiles
 //     share two of their three input rows, which live in a ring of row slots;
 //   - the roles run apart and meet at mbarriers only: warp 17 copies rows
-//     ahead (cp.async) as slots come free; one thread of warp 16 issues a
+//     ahead as slots come free, with 64 channels one TMA box of 128 pixels
+//     and a cp.async of the two halo pixels, with 16 channels cp.async; one
+//     thread of warp 16 issues a
 //     tile's 9 CIN / 16 MMAs (M = 128, N = NOUT, K = 16, BF16 operands) into
 //     one of two TMEM accumulators of NOUT FP32 columns, with tcgen05.commit
 //     signalling the accumulator and the freed row slots; warps 0-7 and 8-15
 //     take the even and the odd tiles' accumulators (tcgen05.ld), give the
 //     accumulator back as soon as it is in registers, apply bias / GELU and
-//     store.
+//     store.  A lane holds 32 outputs of one pixel, so a warp's 16-byte
+//     stores of an NHWC tensor would touch 32 lines each: with 64 channels
+//     the BF16 outputs go through 2 KB of shared memory per warp and a TMA
+//     store, and the pre-activations (FP32, read by the backward pass of the
+//     same kernel only) lie in blocks of 128 pixels, [channel / 4][pixel][4],
+//     where a warp's float4 accesses are contiguous.
 // What bounds it: a 64 -> 64 tile's 36 MMAs take 48 cycles each (each reads
 // 6 KB of operands from shared memory at 128 B per clock; N = 128 would be
 // the first shape that runs at the tensor core's own rate), 1740 cycles, and
@@ -1050,9 +1060,8 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 constexpr int TC_THREADS = 576, TC_TW = 128, TC_RW = TC_TW + 2;
 constexpr int TC_MMA_WARP = 16, TC_COPY_WARP = 17;
 constexpr uint32_t TC_IN_LBO = TC_RW * 16;               // 2080: channel-chunk stride of a staged row
-// Dynamic shared memory requested: the operands need at most 178.7 KB (64 ->
-// 64); the rest is slack so that every address a descriptor can form stays
-// inside the block.
+// Dynamic shared memory requested: 64 -> 64 needs 215 KB; the rest is slack
+// so that every address a descriptor can form stays inside the block.
 constexpr uint32_t TC_SMEM = 220 * 1024;
 constexpr long long TC_WAIT_CYCLES = 2000000000ll;       // about 1 s at 2 GHz
 
@@ -1068,14 +1077,19 @@ struct TcGeom {
     static constexpr uint32_t W_LBO = NOUT * 16;               // chunk stride of one tap's weights (no swizzle)
     static constexpr uint32_t W_TAP = CH * W_LBO;              // one tap: [n][128 B] or [k / 8][n][8]
     static constexpr uint32_t W_BYTES = 9 * W_TAP;
-    static constexpr uint32_t IN_ROW = SW ? (TC_RW * 128 + 1023) / 1024 * 1024  // [column][128 B]
-                                          : CH * TC_IN_LBO;                       // [k / 8][column][8]
+    // A row slot holds columns j0 - 1 .. j0 + 128.  Swizzled: [column][128 B]
+    // with column j0 at a 1024-byte boundary, where the TMA box of 128
+    // columns goes, and a halo column on each side of it.
+    static constexpr uint32_t COL0 = SW ? 1024 - 128 : 0;      // of column j0 - 1 in the slot
+    static constexpr uint32_t IN_ROW = SW ? 1024 + TC_TW * 128 + 1024 : CH * TC_IN_LBO;  // else [k / 8][column][8]
     static constexpr int SLOTS = 6;                              // row ring
     static constexpr uint32_t BAR_OFF = W_BYTES + SLOTS * IN_ROW;  // mbarriers (BAR_*), then the TMEM address
     static constexpr int BAR_FULL = 0, BAR_FREE = SLOTS;         // row slots: copied / read by the MMAs
     static constexpr int BAR_ACC = 2 * SLOTS, BAR_OUT = 2 * SLOTS + 2;  // accumulators: computed / read
     static constexpr int NBAR = 2 * SLOTS + 4;
-    static constexpr uint32_t BIAS_OFF = BAR_OFF + 8 * NBAR + 16;  // NOUT FP32 bias values
+    static constexpr uint32_t BIAS_OFF = BAR_OFF + 8 * NBAR + 16;  // NOUT FP32 bias values, [8][NOUT] column sums
+    static constexpr bool STAGE = NOUT == 64;                    // outputs through shared memory and TMA
+    static constexpr uint32_t STAGE_OFF = (BIAS_OFF + 9 * 4 * NOUT + 1023) / 1024 * 1024;  // [16 warps][32 pixels][64 B]
     static constexpr uint32_t TMEM_COLS = 2 * NOUT < 32 ? 32 : 2 * NOUT;  // two accumulators (allocation >= 32)
     static constexpr int COLS = NOUT / 2;                        // accumulator columns per epilogue warp
     static constexpr int HC = COLS < 16 ? COLS : 16;             // columns taken at once
@@ -1084,7 +1098,7 @@ struct TcGeom {
     // M >> 4 at bit 24.
     static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NOUT >> 3) << 17) |
                                       ((uint32_t)(TC_TW >> 4) << 24);
-    static_assert(BIAS_OFF % 16 == 0 && BIAS_OFF + 9 * 4 * NOUT <= TC_SMEM, "shared memory");
+    static_assert(BIAS_OFF % 16 == 0 && STAGE_OFF + (STAGE ? 16 * 2048 : 0) <= TC_SMEM, "shared memory");
     static_assert(!SW || (W_TAP % 1024 == 0 && W_BYTES % 1024 == 0 && IN_ROW % 1024 == 0), "swizzle atoms");
     static_assert(NOUT % 16 == 0 && CIN % 16 == 0, "shapes");
 };
@@ -1208,7 +1222,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__restrict__ B,
                const float *__restrict__ bias, int nbias, __nv_bfloat16 *__restrict__ out_bf,
                float *__restrict__ z_f32, const float *__restrict__ zprev, int H, int W, int ntiles, int mode,
-               int flip, float *__restrict__ bpart)
+               int flip, int zblk, float *__restrict__ bpart, const __grid_constant__ CUtensorMap mld,
+               const __grid_constant__ CUtensorMap mst)
 {
     using G = TcGeom<CIN, NOUT>;
     constexpr int CH = G::CH, COLS = G::COLS, HC = G::HC, SLOTS = G::SLOTS;
@@ -1235,9 +1250,9 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        // one arrival each: the copying warp's, a commit's, or (an
-        // accumulator read) one per warp of its group
-        for (int b = 0; b < G::BAR_OUT; b++) mbar_init(bar(b), 1);
+        // arrivals: the copying warp's (a TMA box's besides), a commit's, or
+        // (an accumulator read) one per warp of its group
+        for (int b = 0; b < G::BAR_OUT; b++) mbar_init(bar(b), G::SW && b < G::BAR_FREE ? 2 : 1);
         mbar_init(bar(G::BAR_OUT), 8);
         mbar_init(bar(G::BAR_OUT + 1), 8);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1266,19 +1281,35 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
     const int my_tiles = (int)(((long long)(blockIdx.x + 1) * ntiles) / gridDim.x) - t0;
 
     if (warp == TC_COPY_WARP) {
-        // ---- rows: lane l copies channel chunk l % CH of columns l / CH + (32 / CH) m
-        const int kc = lane % CH, px0 = lane / CH;
-        constexpr int STEP = 32 / CH;
-        auto load_row = [&](int seg, int n, int i, int d, int slot) {  // input row i - 1 + d, columns j0 - 1 .. j0 + 128
+        // ---- rows: input row i - 1 + d, columns j0 - 1 .. j0 + 128
+        auto load_row = [&](int seg, int n, int i, int d, int slot) {
             const int j0 = seg * TC_TW;
-            const __nv_bfloat16 *src = in + ((size_t)n * H + wrap(i - 1 + d, H)) * W * CIN + kc * 8;
+            const size_t row = (size_t)n * H + wrap(i - 1 + d, H);
             unsigned char *dst = tc_smem + G::W_BYTES + slot * G::IN_ROW;
-#pragma unroll 8
-            for (int px = px0; px < TC_RW; px += STEP) {
-                const uint32_t off = G::SW ? px * 128 + ((kc ^ (px & 7)) << 4) : kc * TC_IN_LBO + px * 16;
-                int j = j0 + px - 1;
-                j = j < 0 ? j + W : (j >= W ? j - W : j);
-                cp_async16(dst + off, src + (size_t)j * CIN);
+            if constexpr (G::SW) {
+                if (lane == 0) {
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar(G::BAR_FULL + slot)),
+                                 "r"(TC_TW * 128) : "memory");
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes "
+                                 "[%0], [%1, {%2, %3}], [%4];" ::"r"(smem_addr(dst) + 1024), "l"(&mld), "r"(0),
+                                 "r"((int)(row * W + j0)), "r"(bar(G::BAR_FULL + slot)) : "memory");
+                }
+                if (lane < 16) {
+                    // the halo columns: chunk lane % 8 of columns j0 - 1 and j0 + 128
+                    const int c = lane & 7, j = lane < 8 ? (j0 == 0 ? W - 1 : j0 - 1) : (j0 + TC_TW == W ? 0 : j0 + TC_TW);
+                    const uint32_t off = lane < 8 ? G::COL0 + ((c ^ 7) << 4) : 1024 + TC_TW * 128 + (c << 4);
+                    cp_async16(dst + off, in + (row * W + j) * CIN + c * 8);
+                }
+            } else {
+                // lane l copies channel chunk l % CH of columns l / CH + (32 / CH) m
+                const int kc = lane % CH;
+                const __nv_bfloat16 *src = in + row * W * CIN + kc * 8;
+#pragma unroll
+                for (int px = lane / CH; px < TC_RW; px += 32 / CH) {
+                    int j = j0 + px - 1;
+                    j = j < 0 ? j + W : (j >= W ? j - W : j);
+                    cp_async16(dst + kc * TC_IN_LBO + px * 16, src + (size_t)j * CIN);
+                }
             }
         };
         // Row q is announced once its copies are complete; two more rows may
@@ -1343,7 +1374,7 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                     for (int ks = 0; ks < CIN / 16; ks++) {
                         // start-address offsets: the pixel shift (whole 128-byte rows
                         // when swizzled) and the K-slice (32 bytes within the row)
-                        const uint32_t ao = G::SW ? ((1 + dq) * 128 + 32 * ks) >> 4 : ((1 + dq) * 16 + 2 * ks * TC_IN_LBO) >> 4;
+                        const uint32_t ao = G::SW ? (G::COL0 + (1 + dq) * 128 + 32 * ks) >> 4 : ((1 + dq) * 16 + 2 * ks * TC_IN_LBO) >> 4;
                         const uint32_t bo = G::SW ? (tap * G::W_TAP + 32 * ks) >> 4 : (tap * G::W_TAP + 2 * ks * G::W_LBO) >> 4;
                         umma_f16(d, rowdesc[1 + dp] + ao, bdesc0 + bo, G::IDESC, (tap | ks) != 0);
                     }
@@ -1382,8 +1413,11 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
         for (int c = 0; c < (BSUM ? COLS / 2 : 1); c++) bsum[c] = bc2(0.0f);
         int seg = (t0 + grp) / R, r = (t0 + grp) - seg * R;
         for (int k = grp; k < my_tiles; k += 2) {
-            const size_t p = (size_t)r * W + seg * TC_TW + 32 * q + lane;
-            const size_t o = p * NOUT + COLS * h;  // this thread's COLS outputs
+            const size_t p0 = (size_t)r * W + seg * TC_TW;             // the tile's first pixel
+            const size_t o = (p0 + 32 * q + lane) * NOUT + COLS * h;   // this thread's COLS outputs
+            // its pre-activations: four columns each zstep floats from the last
+            const size_t oz = zblk ? p0 * NOUT + COLS * h / 4 * (4 * TC_TW) + (32 * q + lane) * 4 : o;
+            const int zstep = zblk ? 4 * TC_TW : 4;
             r += 2;
             while (r >= R) { r -= R; seg++; }
             // the pre-activations of the backward pass do not depend on the
@@ -1391,7 +1425,7 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
             float4 zp[HC / 4];
             if (mode == 2 && zprev) {
 #pragma unroll
-                for (int c = 0; c < HC / 4; c++) zp[c] = reinterpret_cast<const float4 *>(zprev + o)[c];
+                for (int c = 0; c < HC / 4; c++) zp[c] = *reinterpret_cast<const float4 *>(zprev + oz + c * zstep);
             }
             // the warp-wide TMEM load below needs the whole warp: agree on the outcome
             if (!__all_sync(0xffffffffu, mbar_wait(bar(G::BAR_ACC + grp), (k >> 1) & 1))) break;
@@ -1418,7 +1452,7 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                 if (mode == 2 && zprev) {
                     if (c0 > 0) {
 #pragma unroll
-                        for (int c = 0; c < HC / 4; c++) zp[c] = reinterpret_cast<const float4 *>(zprev + o + c0)[c];
+                        for (int c = 0; c < HC / 4; c++) zp[c] = *reinterpret_cast<const float4 *>(zprev + oz + (c0 / 4 + c) * zstep);
                     }
 #pragma unroll
                     for (int c = 0; c < HC / 4; c++) {
@@ -1434,9 +1468,13 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                         bsum[c0 / 2 + c] = add2(bsum[c0 / 2 + c], fp2{v[2 * c], v[2 * c + 1]});
                 }
                 if (z_f32) {
-                    float4 *zd = reinterpret_cast<float4 *>(z_f32 + o + c0);
+                    // zblk is for the pre-activations of hidden layers (mode 1)
+                    float *zd = z_f32 + (mode == 1 ? oz : o);
+                    const int st = mode == 1 ? zstep : 4;
 #pragma unroll
-                    for (int c = 0; c < HC / 4; c++) zd[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                    for (int c = 0; c < HC / 4; c++)
+                        *reinterpret_cast<float4 *>(zd + (c0 / 4 + c) * st) =
+                            make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
                 }
                 if (mode == 1) {
 #pragma unroll
@@ -1446,9 +1484,35 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                         v[2 * c + 1] = gv.y;
                     }
                 }
-                store_bf16<HC>(out_bf + o + c0, v);
+                if constexpr (G::STAGE) {
+                    // [pixel][64 B] in the 64-byte swizzle (16-byte chunk XOR bits 7-8 of
+                    // the address); the warp's last TMA store has read it before
+                    if (c0 == 0) {
+                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        __syncwarp();
+                    }
+                    unsigned char *sp = tc_smem + G::STAGE_OFF + warp * 2048 + lane * 64;
+#pragma unroll
+                    for (int c = 0; c < HC / 8; c++)
+                        *reinterpret_cast<uint4 *>(sp + (((c0 / 8 + c) ^ ((lane >> 1) & 3)) << 4)) =
+                            make_uint4(pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
+                                       pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
+                } else {
+                    store_bf16<HC>(out_bf + o + c0, v);
+                }
+            }
+            if constexpr (G::STAGE) {
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(&mst),
+                                 "r"(COLS * h), "r"((int)(p0 + 32 * q)), "r"(sbase + G::STAGE_OFF + warp * 2048) : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
             }
         }
+        if (G::STAGE && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        __syncwarp();
         if constexpr (BSUM) {
             // the sum over the lanes of a warp
             float *sb = bias_s + NOUT;  // [8 = (group, pixel quarter)][NOUT]
@@ -1518,7 +1582,7 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st)
         if (e != cudaSuccess) { sms = 0; return e; }
     }
     if constexpr ((CIN == 16 || CIN == 64) && (NOUT == 16 || NOUT == 64)) {
-        if (a.W % TC_TW == 0 && a.npix % (a.H * a.W) == 0 && use_tc()) {
+        if (a.W % TC_TW == 0 && a.npix % (a.H * a.W) == 0 && use_tc() && (CIN != 64 || a.ld) && (NOUT != 64 || a.st)) {
             static bool tc_ready = false;
             if (!tc_ready) {
                 cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<CIN, NOUT, false>,
@@ -1532,12 +1596,14 @@ cudaError_t launch_conv_t(const ConvArgs &a, cudaStream_t st)
             const int ntiles = a.npix / TC_TW;
             const int blocks = ntiles < sms ? ntiles : sms;
             float *z = a.keep_z ? a.z : nullptr;
+            const CUtensorMap none{};
+            const CUtensorMap &ld = a.ld ? *a.ld : none, &st_map = a.st ? *a.st : none;
             if (a.bpart)
                 conv_tc_kernel<CIN, NOUT, true><<<blocks, TC_THREADS, TC_SMEM, st>>>(
-                    a.in, a.B, a.bias, a.nbias, a.out, z, a.zprev, a.H, a.W, ntiles, a.mode, a.flip, a.bpart);
+                    a.in, a.B, a.bias, a.nbias, a.out, z, a.zprev, a.H, a.W, ntiles, a.mode, a.flip, a.zblk, a.bpart, ld, st_map);
             else
                 conv_tc_kernel<CIN, NOUT, false><<<blocks, TC_THREADS, TC_SMEM, st>>>(
-                    a.in, a.B, a.bias, a.nbias, a.out, z, a.zprev, a.H, a.W, ntiles, a.mode, a.flip, nullptr);
+                    a.in, a.B, a.bias, a.nbias, a.out, z, a.zprev, a.H, a.W, ntiles, a.mode, a.flip, a.zblk, nullptr, ld, st_map);
             if (a.bpart) *a.nb = blocks;
             return cudaGetLastError();
         }
@@ -1610,7 +1676,37 @@ struct hlbm_sur {
     float *bpart = nullptr;  // partial bias gradients, BIAS_BLOCKS rows of MAXC
     int last_batch = 0;
     int64_t adam_t = 0;
+    // Tensor maps of the BF16 buffers as [pixel][64]: boxes of 128 pixels x 64
+    // channels (row loads) and 32 x 32 (stores) of the tcgen05 kernel.
+    struct Maps {
+        CUtensorMap ld, st;
+    };
+    Maps amap[MAX_LAYERS + 1], gmap[2];
+    bool maps = false;  // the maps are there
+    bool zblk = false;  // every layer runs on the tcgen05 kernel: z in blocks of 128 pixels
 };
+
+// The tensor maps of one [npix][64] BF16 buffer; false if the driver has none.
+static bool encode_conv_maps(void *buf, size_t npix, hlbm_sur::Maps *m)
+{
+    static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+    if (!encode) {
+        cudaDriverEntryPointQueryResult q;
+        void *fn = nullptr;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess || !fn)
+            return false;
+        encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    }
+    const cuuint64_t dims[2] = {64, npix}, strides[1] = {128};
+    const cuuint32_t estr[2] = {1, 1}, box_ld[2] = {64, TC_TW}, box_st[2] = {32, 32};
+    return encode(&m->ld, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, buf, dims, strides, box_ld, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
+           encode(&m->st, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, buf, dims, strides, box_st, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 extern "C" {
 
@@ -1680,6 +1776,17 @@ int hlbm_sur_create(int nlayer, const int *widths, int H, int W, int batch_max, 
     }
     if (ok) ok = cudaMalloc(&s->act[nlayer], npix * s->cpad_out[nlayer - 1] * 2) == cudaSuccess;
     if (!ok) { cudaGetLastError(); hlbm_sur_destroy(s); return HLBM_ERR_NOMEM; }
+    if (W % TC_TW == 0 && use_tc()) {
+        // (a buffer of 16 channels has no map; gbuf holds MAXC channels)
+        s->maps = encode_conv_maps(s->gbuf[0], npix, &s->gmap[0]) && encode_conv_maps(s->gbuf[1], npix, &s->gmap[1]);
+        s->zblk = s->maps;
+        for (int l = 0; l < nlayer; l++) {
+            if (s->cpad_in[l] == 64) s->maps = s->maps && encode_conv_maps(s->act[l], npix, &s->amap[l]);
+            for (int c : {s->cpad_in[l], s->cpad_out[l]}) s->zblk = s->zblk && (c == 16 || c == 64);
+        }
+        if (s->cpad_out[nlayer - 1] == 64) s->maps = s->maps && encode_conv_maps(s->act[nlayer], npix, &s->amap[nlayer]);
+        s->zblk = s->zblk && s->maps;
+    }
     if (cudaMemsetAsync(s->m, 0, off * 4, s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->v, 0, off * 4, s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->p, 0, off * 4, s->stream) != cudaSuccess) {
@@ -1740,8 +1847,11 @@ static int sur_run(hlbm_sur *s, const float *x, float *y, int B, bool keep_z)
     if (cudaGetLastError() != cudaSuccess) return HLBM_ERR_CUDA;
     for (int l = 0; l < s->L; l++) {
         const bool last = l == s->L - 1;
-        const ConvArgs a{s->act[l], s->Wb[l], s->p + s->boff[l], s->width[l + 1], s->act[l + 1],
-                         (keep_z || last) ? s->z[l] : nullptr, nullptr, npix, s->H, s->W, last ? 0 : 1, 0};
+        ConvArgs a{s->act[l], s->Wb[l], s->p + s->boff[l], s->width[l + 1], s->act[l + 1],
+                   (keep_z || last) ? s->z[l] : nullptr, nullptr, npix, s->H, s->W, last ? 0 : 1, 0};
+        a.ld = s->maps ? &s->amap[l].ld : nullptr;
+        a.st = s->maps ? &s->amap[l + 1].st : nullptr;
+        a.zblk = s->zblk;
         if (launch_conv(s->cpad_in[l], s->cpad_out[l], a, s->stream) != cudaSuccess) return HLBM_ERR_CUDA;
     }
     residual_loss_kernel<<<1024, 256, 0, s->stream>>>(s->xin, s->z[s->L - 1], s->cpad_out[s->L - 1], nullptr,
@@ -1819,8 +1929,10 @@ static int sur_backward(hlbm_sur *s, const float *target, const float *dy, int a
             if (dx) {
                 // the network's part of dL/dx: W_0^T * dz_0, the transposed
                 // convolution without GELU' (the input has no activation)
-                const ConvArgs a{s->gbuf[gb], s->Wd[0], nullptr, 0, s->gbuf[gb ^ 1], dzf[cur ^ 1], nullptr, npix,
-                                 s->H, s->W, 2, 1};
+                ConvArgs a{s->gbuf[gb], s->Wd[0], nullptr, 0, s->gbuf[gb ^ 1], dzf[cur ^ 1], nullptr, npix,
+                           s->H, s->W, 2, 1};
+                a.ld = s->maps ? &s->gmap[gb].ld : nullptr;
+                a.st = s->maps ? &s->gmap[gb ^ 1].st : nullptr;
                 if (launch_conv(s->cpad_out[0], s->cpad_in[0], a, s->stream) != cudaSuccess) return HLBM_ERR_CUDA;
                 gather_grad_kernel<<<1024, 256, 0, s->stream>>>(dzf[cur ^ 1], s->cpad_in[0], s->width[0], npix, 1, dx);
                 if (cudaGetLastError() != cudaSuccess) return HLBM_ERR_CUDA;
@@ -1836,6 +1948,9 @@ static int sur_backward(hlbm_sur *s, const float *target, const float *dy, int a
         a.bpart = s->bpart;
         a.nb = &nb;
         a.keep_z = false;
+        a.ld = s->maps ? &s->gmap[gb].ld : nullptr;
+        a.st = s->maps ? &s->gmap[gb ^ 1].st : nullptr;
+        a.zblk = s->zblk;
         if (launch_conv(s->cpad_out[l], s->cpad_in[l], a, s->stream) != cudaSuccess) return HLBM_ERR_CUDA;
         cur ^= 1;
         gb ^= 1;
