@@ -1034,7 +1034,10 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 //     thread of warp 16 issues a
 //     tile's 9 CIN / 16 MMAs (M = 128, N = NOUT, K = 16, BF16 operands) into
 //     one of two TMEM accumulators of NOUT FP32 columns, with tcgen05.commit
-//     signalling the accumulator and the freed row slots; warps 0-7 and 8-15
+//     signalling the accumulator; the tensor core takes an MMA only two or so
+//     ahead, so whatever this thread waits for leaves it idle, and warp 18
+//     does the waiting (rows copied, accumulator read) and counts the tiles
+//     that may start; warps 0-7 and 8-15
 //     take the even and the odd tiles' accumulators (tcgen05.ld), give the
 //     accumulator back as soon as it is in registers, apply bias / GELU and
 //     store.  A lane holds 32 outputs of one pixel, so a warp's 16-byte
@@ -1049,7 +1052,7 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 // its GELUs 1024 cycles of the MUFU (two per value).  With all warps in one
 // loop behind a barrier per tile, the copy, the TMEM read, the GELU and the
 // stores of a tile stood one after another and a tile took 4500 cycles: 133
-// us per 64 -> 64 layer of 16 x 256^2, against @NEW@ with the roles apart.
+// us per 64 -> 64 layer of 16 x 256^2, against 80 us with the roles apart.
 // Operands are K-major.  With 64 channels a pixel (or a weight row) is one
 // 128-byte row of the 128-byte swizzle layout, so a tap's pixel shift moves
 // the operand by whole aligned rows.  With 16 channels they use the layout
@@ -1057,8 +1060,8 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 // 8-row groups SBO = 128 bytes apart (consecutive pixels are consecutive
 // 16-byte rows and a pixel shift is a 16-byte offset of the start
 // address), the two 8-channel halves of a K-slice LBO bytes apart.
-constexpr int TC_THREADS = 576, TC_TW = 128, TC_RW = TC_TW + 2;
-constexpr int TC_MMA_WARP = 16, TC_COPY_WARP = 17;
+constexpr int TC_THREADS = 608, TC_TW = 128, TC_RW = TC_TW + 2;
+constexpr int TC_MMA_WARP = 16, TC_COPY_WARP = 17, TC_READY_WARP = 18;
 constexpr uint32_t TC_IN_LBO = TC_RW * 16;               // 2080: channel-chunk stride of a staged row
 // Dynamic shared memory requested: 64 -> 64 needs 215 KB; the rest is slack
 // so that every address a descriptor can form stays inside the block.
@@ -1087,6 +1090,7 @@ struct TcGeom {
     static constexpr int BAR_FULL = 0, BAR_FREE = SLOTS;         // row slots: copied / read by the MMAs
     static constexpr int BAR_ACC = 2 * SLOTS, BAR_OUT = 2 * SLOTS + 2;  // accumulators: computed / read
     static constexpr int NBAR = 2 * SLOTS + 4;
+    static constexpr uint32_t READY_OFF = BAR_OFF + 8 * NBAR + 8;  // tiles whose MMAs may be issued
     static constexpr uint32_t BIAS_OFF = BAR_OFF + 8 * NBAR + 16;  // NOUT FP32 bias values, [8][NOUT] column sums
     static constexpr bool STAGE = NOUT == 64;                    // outputs through shared memory and TMA
     static constexpr uint32_t STAGE_OFF = (BIAS_OFF + 9 * 4 * NOUT + 1023) / 1024 * 1024;  // [16 warps][32 pixels][64 B]
@@ -1211,6 +1215,29 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
+__device__ __forceinline__ void st_release(uint32_t addr, int v)
+{
+    asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire(uint32_t addr)
+{
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+// Bounded wait for a counter in shared memory to exceed k, as mbar_wait.
+__device__ __forceinline__ bool count_wait(uint32_t addr, int k)
+{
+    if (ld_acquire(addr) > k) return true;
+    const long long t0 = clock64();
+    while (ld_acquire(addr) <= k) {
+        if (clock64() - t0 > TC_WAIT_CYCLES) {
+            atomicExch(&g_tc_status, 1);
+            return false;
+        }
+    }
+    return true;
+}
 __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -1232,6 +1259,7 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
     const uint32_t w_s = sbase, ring_s = sbase + G::W_BYTES;
     auto bar = [&](int b) { return sbase + G::BAR_OFF + 8 * b; };
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tc_smem + G::BAR_OFF + 8 * G::NBAR);
+    const uint32_t ready_s = sbase + G::READY_OFF;
     float *bias_s = reinterpret_cast<float *>(tc_smem + G::BIAS_OFF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nseg = W / TC_TW;
@@ -1255,6 +1283,7 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
         for (int b = 0; b < G::BAR_OUT; b++) mbar_init(bar(b), G::SW && b < G::BAR_FREE ? 2 : 1);
         mbar_init(bar(G::BAR_OUT), 8);
         mbar_init(bar(G::BAR_OUT + 1), 8);
+        st_release(ready_s, 0);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // weights of all taps: B[tap][n][k] -> [tap][k / 8][n][8]
@@ -1380,22 +1409,29 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                     }
                 }
             };
-            bool ok = true;
-            int q0 = 0, q = 0;  // the tile's first row; rows known to be copied
-            int i = t0 % H;
-            for (int k = 0; k < my_tiles && ok; k++) {
-                const bool last = k + 1 == my_tiles || i == H - 1;  // of its run
-                if (k >= 2) ok = mbar_wait(bar(G::BAR_OUT + (k & 1)), ((k >> 1) - 1) & 1);
-                for (; ok && q < q0 + 3; q++) ok = mbar_wait(bar(G::BAR_FULL + q % SLOTS), (q / SLOTS) & 1);
-                if (!ok) break;
+            int q0 = 0, i = t0 % H;  // the tile's first row
+            for (int k = 0; k < my_tiles; k++) {
+                if (!count_wait(ready_s, k)) break;
                 tc_fence_after();
                 if (flip) issue(tmem + (k & 1) * NOUT, q0, true);
                 else issue(tmem + (k & 1) * NOUT, q0, false);
                 umma_commit(bar(G::BAR_ACC + (k & 1)));
-                for (int e = 0; e < (last ? 3 : 1); e++) umma_commit(bar(G::BAR_FREE + (q0 + e) % SLOTS));
-                if (k + 1 == my_tiles)  // no arrival may be outstanding when the CTA ends
-                    for (int e = 0; e < 3; e++) mbar_wait(bar(G::BAR_FREE + (q0 + e) % SLOTS), ((q0 + e) / SLOTS) & 1);
-                q0 += last ? 3 : 1;
+                q0 += i == H - 1 ? 3 : 1;
+                i = i == H - 1 ? 0 : i + 1;
+            }
+        }
+        __syncwarp();
+    } else if (warp == TC_READY_WARP) {
+        if (lane == 0) {
+            // ---- tile k may start once its rows are copied and its accumulator
+            // has been read (tile k - 2)
+            bool ok = true;
+            int q0 = 0, q = 0, i = t0 % H;  // the tile's first row; rows known to be copied
+            for (int k = 0; k < my_tiles && ok; k++) {
+                for (; ok && q < q0 + 3; q++) ok = mbar_wait(bar(G::BAR_FULL + q % SLOTS), (q / SLOTS) & 1);
+                if (ok && k >= 2) ok = mbar_wait(bar(G::BAR_OUT + (k & 1)), ((k >> 1) - 1) & 1);
+                if (ok) st_release(ready_s, k + 1);
+                q0 += i == H - 1 ? 3 : 1;
                 i = i == H - 1 ? 0 : i + 1;
             }
         }
@@ -1412,6 +1448,9 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
 #pragma unroll
         for (int c = 0; c < (BSUM ? COLS / 2 : 1); c++) bsum[c] = bc2(0.0f);
         int seg = (t0 + grp) / R, r = (t0 + grp) - seg * R;
+        // the tile's first row and its place in the image (the group's first
+        // warp gives the row slots back)
+        int q0 = grp == 0 ? 0 : (t0 % H == H - 1 ? 3 : 1), i = (t0 + grp) % H;
         for (int k = grp; k < my_tiles; k += 2) {
             const size_t p0 = (size_t)r * W + seg * TC_TW;             // the tile's first pixel
             const size_t o = (p0 + 32 * q + lane) * NOUT + COLS * h;   // this thread's COLS outputs
@@ -1430,6 +1469,17 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
             // the warp-wide TMEM load below needs the whole warp: agree on the outcome
             if (!__all_sync(0xffffffffu, mbar_wait(bar(G::BAR_ACC + grp), (k >> 1) & 1))) break;
             tc_fence_after();
+            if ((warp & 7) == 0) {
+                // the tile's MMAs (and those before them) are done: its first row
+                // is free, all three if no later tile of the run shares them
+                const bool last = k + 1 == my_tiles || i == H - 1;
+                if (lane < (last ? 3 : 1)) mbar_arrive(bar(G::BAR_FREE + (q0 + lane) % SLOTS));
+                __syncwarp();
+                for (int e = 0; e < 2; e++) {
+                    q0 += i == H - 1 ? 3 : 1;
+                    i = i == H - 1 ? 0 : i + 1;
+                }
+            }
 #pragma unroll
             for (int c0 = 0; c0 < COLS; c0 += HC) {
                 float v[HC];
