@@ -21,6 +21,7 @@
 #include "hlbm_device.cuh"
 #include "hlbm_tma.cuh"
 #include "hlbm_march.cuh"
+#include "hlbm_split.cuh"
 
 using namespace hlbm;
 
@@ -71,7 +72,9 @@ struct hlbm_handle {
     bool moments = false;       // HLBM_FP32_MOMENTS: 7 FP32 planes, moment-state kernel
     bool walls = false;         // a wall side: tiled kernel plus wall_ghost_kernel each step
     bool periodic = false;      // all four sides periodic and ny >= 4 (specialised marching kernels)
-    bool mcache = false;        // FP64 marching: level-n rho, u, theta planes behind the state (A_RHO .. A_TH)
+    bool mcache = false;        // FP64 marching and two-pass forms: level-n rho, u, theta planes behind the state (A_RHO .. A_TH)
+    bool split = false;         // FP64 two-pass form (hlbm_split.cuh)
+    double *split_buf = nullptr;  // its planes between the passes, behind the staging planes
     void *wall_g = nullptr;     // wall ghost rows (KParams::wall_g)
     int march_nseg = 1;         // row segments per strip
     int *d_err = nullptr;       // device-side timeout flag of the TMA kernel
@@ -118,8 +121,8 @@ static size_t payload_bytes(const hlbm_handle *h)
     return h->moments ? h->plane * MS_NPLANE * sizeof(float) : h->plane * (9 * h->fsize + 4 * h->asize);
 }
 
-// Bytes allocated per state copy: the payload, then the FP64 marching
-// form's cache planes.
+// Bytes allocated per state copy: the payload, then the cache planes of the
+// FP64 marching and two-pass forms.
 static size_t alloc_bytes(const hlbm_handle *h)
 {
     return payload_bytes(h) + (h->mcache ? h->plane * A_NCACHE * sizeof(double) : 0);
@@ -129,13 +132,90 @@ static size_t alloc_bytes(const hlbm_handle *h)
 // F(n) and s(n), after init or a checkpoint set the state.
 static cudaError_t fill_cache(hlbm_handle *h)
 {
-    if (!h->mcache) return cudaSuccess;
+    if (!h->mcache || h->split) return cudaSuccess;
     const int blk = 256;
     const long long n = (long long)h->p.nx * h->p.ny;
     const int grid = (int)std::min<long long>((n + blk - 1) / blk, 65535);
     cache_macros_kernel<<<grid, blk, 0, h->stream>>>(pop_planes<double, FullStore<double>>(h, h->cur),
                                                      aux_planes<double, FullStore<double>>(h, h->cur), h->kp);
     return cudaGetLastError();
+}
+
+// FP64 two-pass form: one thread per cell, 32 columns wide.  Few cells are
+// spread over as many SMs as they reach, one warp per CTA: an SM's FP64 pipe
+// takes a warp instruction every 19 cycles from four warps or more, and every
+// 64 cycles from one, however few of its lanes are active.  Many cells run 8
+// rows per CTA.
+static void split_shape(const hlbm_handle *h, dim3 *grid, dim3 *blk)
+{
+    const long long warps = (long long)((h->p.nx + 31) / 32) * h->p.ny;
+    const int rows = warps >= 8 * 1216 ? 8 : (warps >= 4 * 304 ? 4 : 1);
+    *blk = dim3(32, rows);
+    *grid = dim3((h->p.nx + 31) / 32, (h->p.ny + rows - 1) / rows);
+}
+
+// outA: the auxiliary planes the step writes.
+static SplitPlanes split_planes(const hlbm_handle *h, double *outA)
+{
+    double *b = h->split_buf;
+    const size_t P = h->plane;
+    SplitPlanes sp{b, b + P, b + 2 * P, b + 3 * P, b + 4 * P, b + 5 * P, b + 6 * P, b + 7 * P,
+                   outA + A_RHO * P, outA + A_UX * P, outA + A_UY * P, outA + A_TH * P,
+                   2.0 * h->kp.mu, -0.5 * h->kp.mu, 0.25 * h->kp.mu, 0.5 * h->kp.two_minus_gamma, 1.0 - h->kp.sigma};
+    if (!h->mcache) {
+        sp.rho = b + 8 * P; sp.ux = b + 9 * P; sp.uy = b + 10 * P; sp.th = b + 11 * P;
+    }
+    return sp;
+}
+
+static bool any_dirichlet(const hlbm_handle *h)
+{
+    for (int k = 0; k < 4; k++)
+        if (h->p.bc[k] == HLBM_BC_DIRICHLET) return true;
+    return false;
+}
+
+// FP64 two-pass form: what the first level pass reads beside F, s and a1,
+// from state copy cur; `derive`: the cache planes too.
+static cudaError_t split_prepare(hlbm_handle *h, bool derive)
+{
+    if (!h->split) return cudaSuccess;
+    dim3 grid, blk;
+    split_shape(h, &grid, &blk);
+    const double *F = pop_planes<double, FullStore<double>>(h, h->cur);
+    double *A = aux_planes<double, FullStore<double>>(h, h->cur);
+    const SplitPlanes sp = split_planes(h, A);
+    if (any_dirichlet(h)) {
+        if (derive) split_prepare_kernel<true, true><<<grid, blk, 0, h->stream>>>(F, A, sp, h->kp);
+        else split_prepare_kernel<true, false><<<grid, blk, 0, h->stream>>>(F, A, sp, h->kp);
+    } else {
+        if (derive) split_prepare_kernel<false, true><<<grid, blk, 0, h->stream>>>(F, A, sp, h->kp);
+        else split_prepare_kernel<false, false><<<grid, blk, 0, h->stream>>>(F, A, sp, h->kp);
+    }
+    return cudaGetLastError();
+}
+
+template <bool SIG, bool PHI0, bool DIR>
+static cudaError_t launch_split_t(hlbm_handle *h)
+{
+    dim3 grid, blk;
+    split_shape(h, &grid, &blk);
+    const int a = h->cur, b = h->cur ^ 1;
+    using S = FullStore<double>;
+    double *outF = pop_planes<double, S>(h, b), *outA = aux_planes<double, S>(h, b);
+    const SplitPlanes sp = split_planes(h, outA);
+    split_level_kernel<SIG, PHI0, DIR><<<grid, blk, 0, h->stream>>>(pop_planes<double, S>(h, a), aux_planes<double, S>(h, a),
+                                                                    outA, sp, h->kp);
+    if (h->mcache) split_collide_kernel<SIG, DIR, false><<<grid, blk, 0, h->stream>>>(outF, outA, sp, h->kp);
+    else split_collide_kernel<SIG, DIR, true><<<grid, blk, 0, h->stream>>>(outF, outA, sp, h->kp);
+    return cudaGetLastError();
+}
+
+template <bool DIR>
+static cudaError_t launch_split(hlbm_handle *h)
+{
+    if (h->kp.sigma_nonzero) return h->kp.phi_mode == 0 ? launch_split_t<true, true, DIR>(h) : launch_split_t<true, false, DIR>(h);
+    return h->kp.phi_mode == 0 ? launch_split_t<false, true, DIR>(h) : launch_split_t<false, false, DIR>(h);
 }
 
 // Call fn(Types<T, S>{}) for the handle's precision.
@@ -458,6 +538,7 @@ static cudaError_t launch_wall_ghosts(hlbm_handle *h)
 static cudaError_t launch_one_step(hlbm_handle *h)
 {
     if (h->moments) return launch_moments(h);
+    if (h->split) return any_dirichlet(h) ? launch_split<true>(h) : launch_split<false>(h);
     if (h->walls) {
         const cudaError_t e = launch_wall_ghosts(h);
         if (e != cudaSuccess) return e;
@@ -654,15 +735,18 @@ int hlbm_create(const hlbm_params *params, void *stream, hlbm_handle **out)
     h->fsize = (params->precision == HLBM_FP32_F16POP || params->precision == HLBM_FP32_BF16POP) ? 2 : h->asize;
     h->pitch = (params->nx + 31) / 32 * 32;
     h->plane = (size_t)h->pitch * params->ny;
-    // FP64 without wall sides may take the marching kernel (decided below);
-    // its cache planes are allocated up front and dropped from use if not
+    // FP64 without wall sides takes the two-pass form or, with HLBM_MARCH
+    // set, the marching or tiled kernel (decided below); the cache planes are
+    // allocated up front and dropped from use by the tiled kernel
     bool wall_side = false;
     for (int k = 0; k < 4; k++) wall_side = wall_side || params->bc[k] == HLBM_BC_WALL;
     h->mcache = params->precision == HLBM_FP64 && !wall_side;
     const size_t bytes = alloc_bytes(h);
     const size_t ncell = (size_t)params->nx * params->ny;
+    const bool two_pass = h->mcache && !getenv("HLBM_MARCH");
+    const size_t staging = 9 * ncell + (two_pass ? SPLIT_NPLANE_CANON * h->plane + 16 : 0);
     if (cudaMalloc(&h->state[0], bytes) != cudaSuccess || cudaMalloc(&h->state[1], bytes) != cudaSuccess ||
-        cudaMalloc(&h->staging, 9 * ncell * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(&h->staging, staging * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&h->diag_partial, DIAG_BLOCKS * DIAG_NV * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&h->diag_out, DIAG_NV * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&h->d_err, sizeof(int)) != cudaSuccess) {
@@ -715,6 +799,20 @@ int hlbm_create(const hlbm_params *params, void *stream, hlbm_handle **out)
             hlbm_destroy(h);
             return HLBM_ERR_CUDA;
         }
+        *out = h;
+        return HLBM_OK;
+    }
+    // FP64: the two-pass form at every size (1024^2 vortex 377 us per step
+    // against 764 on the marching kernel; Sod tube 400 x 4 19 us against 39
+    // on the tiled kernel).  HLBM_MARCH=<k> picks a marching variant, -1 the
+    // tiled kernel, as for the other precisions.
+    if (two_pass) {
+        h->march_variant = -1;
+        h->split = true;
+        // checkpoints carry the cache planes on the grids whose marching form
+        // does, and hold 13 planes on smaller ones, as with the tiled kernel
+        h->mcache = (long long)params->nx * params->ny > kMarchMinCells;
+        h->split_buf = h->staging + (9 * ncell + 15) / 16 * 16;
         *out = h;
         return HLBM_OK;
     }
@@ -821,6 +919,7 @@ int hlbm_init_fields(hlbm_handle *h, const double *rho, const double *ux, const 
        }), "init_kernel");
     h->cur = 0;
     CK(fill_cache(h), "cache_macros_kernel");
+    CK(split_prepare(h, true), "split_prepare_kernel");
     h->step = 0;
     h->initialized = true;
     CK(cudaStreamSynchronize(h->stream), "init sync");
@@ -1027,6 +1126,7 @@ int hlbm_set_state(hlbm_handle *h, const void *buf, size_t bytes)
     for (int i = 0; i < 9; i++) h->kp.f_ref[i] = hd.ref[i];
     h->cur = 0;
     if (!copy_cache) CK(fill_cache(h), "cache_macros_kernel");
+    CK(split_prepare(h, !copy_cache), "split_prepare_kernel");
     CK(cudaStreamSynchronize(h->stream), "state sync");
     h->step = hd.step;
     h->initialized = true;
