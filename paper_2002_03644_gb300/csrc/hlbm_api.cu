@@ -27,7 +27,7 @@ using namespace hlbm;
 
 namespace {
 
-constexpr int TX64 = 32, TY64 = 8, NT64 = 256;   // FP64 tile
+constexpr int kSms = 152;  // SMs of a GB300 (work is cut for them; any count is correct)
 constexpr int DIAG_BLOCKS = 2 * 152;
 constexpr uint64_t STATE_MAGIC = 0x31305453424c4848ull;  // "HHLBST01"
 
@@ -141,6 +141,20 @@ static cudaError_t fill_cache(hlbm_handle *h)
     return cudaGetLastError();
 }
 
+// Launch of a step kernel that may be set up while the kernel before it on
+// the stream ends (the kernel begins with step_begin()).
+template <typename... K, typename... A>
+static cudaError_t launch_chained(void (*kernel)(K...), dim3 grid, dim3 blk, size_t smem, cudaStream_t stream, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = blk; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // FP64 two-pass form: one thread per cell, 32 columns wide.  Few cells are
 // spread over as many SMs as they reach, one warp per CTA: an SM's FP64 pipe
 // takes a warp instruction every 19 cycles from four warps or more, and every
@@ -204,11 +218,12 @@ static cudaError_t launch_split_t(hlbm_handle *h)
     using S = FullStore<double>;
     double *outF = pop_planes<double, S>(h, b), *outA = aux_planes<double, S>(h, b);
     const SplitPlanes sp = split_planes(h, outA);
-    split_level_kernel<SIG, PHI0, DIR><<<grid, blk, 0, h->stream>>>(pop_planes<double, S>(h, a), aux_planes<double, S>(h, a),
-                                                                    outA, sp, h->kp);
-    if (h->mcache) split_collide_kernel<SIG, DIR, false><<<grid, blk, 0, h->stream>>>(outF, outA, sp, h->kp);
-    else split_collide_kernel<SIG, DIR, true><<<grid, blk, 0, h->stream>>>(outF, outA, sp, h->kp);
-    return cudaGetLastError();
+    const cudaError_t e = launch_chained(split_level_kernel<SIG, PHI0, DIR>, grid, blk, 0, h->stream,
+                                         (const double *)pop_planes<double, S>(h, a), (const double *)aux_planes<double, S>(h, a),
+                                         outA, sp, h->kp);
+    if (e != cudaSuccess) return e;
+    if (h->mcache) return launch_chained(split_collide_kernel<SIG, DIR, false>, grid, blk, 0, h->stream, outF, outA, sp, h->kp);
+    return launch_chained(split_collide_kernel<SIG, DIR, true>, grid, blk, 0, h->stream, outF, outA, sp, h->kp);
 }
 
 template <bool DIR>
@@ -243,16 +258,22 @@ static cudaError_t launch_step(hlbm_handle *h)
     }
     dim3 grid((h->p.nx + TX - 1) / TX, (h->p.ny + TY - 1) / TY);
     const int a = h->cur, b = h->cur ^ 1;
-    fused_step_kernel<T, S, TX, TY, NT><<<grid, NT, Geo::smem_bytes, h->stream>>>(
-        pop_planes<T, S>(h, a), aux_planes<T, S>(h, a), pop_planes<T, S>(h, b), aux_planes<T, S>(h, b), h->kp);
-    return cudaGetLastError();
+    return launch_chained(fused_step_kernel<T, S, TX, TY, NT>, grid, NT, Geo::smem_bytes, h->stream,
+                          (const typename S::raw *)pop_planes<T, S>(h, a), (const T *)aux_planes<T, S>(h, a),
+                          pop_planes<T, S>(h, b), aux_planes<T, S>(h, b), h->kp);
 }
 
-// Tiled FP32 kernels (HLBM_MARCH=-1).  Grids of up to 2048^2 cells use the
-// plain tiled kernel with 32x32 tiles and larger grids the persistent TMA
-// kernel with 32x16 tiles.  HLBM_FP32_TMA=<k> forces TMA tile k,
-// HLBM_FP32_TMA=-1 the plain kernel with HLBM_FP32_TILE=<k> (tuning sweeps).
-constexpr int kNumFp32Tiles = 5;  // plain: 32x16x256, 64x16x256, 32x8x128, 64x32x512, 32x32x512
+// Tiled FP32 kernels (grids up to 768^2, wall sides, HLBM_MARCH=-1).  The
+// plain tiled kernel has 16x16 tiles with 512 threads, so that no thread has
+// more than one cell in any phase: a step of a small grid is a chain of
+// trips to memory and of the phases' latencies, which 32x32 tiles walked two
+// or three times on a part of the SMs (per step, 32x32 -> 16x16: 128^2 12.2 ->
+// 5.4 us, 256^2 11.9 -> 5.8, 512^2 15.6 -> 12.0, 768^2 24.7 -> 22.5, two walls at
+// 1500 x 900 63 -> 54).  Grids above 2048^2 cells take the persistent TMA
+// kernel with 32x16 tiles where HLBM_MARCH=-1 asks for tiles.
+// HLBM_FP32_TMA=<k> forces TMA tile k, HLBM_FP32_TMA=-1 the plain kernel with
+// HLBM_FP32_TILE=<k> (tuning sweeps).
+constexpr int kNumFp32Tiles = 6;  // plain: 32x16x256, 64x16x256, 32x8x128, 64x32x512, 32x32x512, 16x16x512
 constexpr int kNumTma = 4;        // TMA: 32x16x512, 32x16x256, 64x16x512, 32x32x512
 
 static int env_choice(const char *name, int dflt, int lo, int hi)
@@ -338,7 +359,7 @@ static cudaError_t setup_fp32_kernel(hlbm_handle *h)
 {
     const bool large = (long long)h->p.nx * h->p.ny > 2048ll * 2048ll;
     h->tma_variant = env_choice("HLBM_FP32_TMA", large ? 0 : -1, -1, kNumTma);
-    h->tile_variant = env_choice("HLBM_FP32_TILE", 4, 0, kNumFp32Tiles);
+    h->tile_variant = env_choice("HLBM_FP32_TILE", 5, 0, kNumFp32Tiles);
     switch (h->tma_variant) {
     case -1: return cudaSuccess;
     case 1: return prepare_tma<32, 16, 256>(h);
@@ -425,14 +446,13 @@ static cudaError_t launch_pair(hlbm_handle *h)
     T *outA = aux_planes<T, S>(h, b);
     const bool sig = h->kp.sigma_nonzero != 0, phi0 = h->kp.phi_mode == 0;
     if (sig && phi0)
-        march_pair_kernel<T, S, NT, MINB, true, true, PER><<<grid, NT, G::smem_bytes, h->stream>>>(inF, inA, outF, outA, h->kp, h->march_nseg);
+        return launch_chained(march_pair_kernel<T, S, NT, MINB, true, true, PER>, grid, NT, G::smem_bytes, h->stream, inF, inA, outF, outA, h->kp, h->march_nseg);
     else if (sig)
-        march_pair_kernel<T, S, NT, MINB, true, false, PER><<<grid, NT, G::smem_bytes, h->stream>>>(inF, inA, outF, outA, h->kp, h->march_nseg);
+        return launch_chained(march_pair_kernel<T, S, NT, MINB, true, false, PER>, grid, NT, G::smem_bytes, h->stream, inF, inA, outF, outA, h->kp, h->march_nseg);
     else if (phi0)
-        march_pair_kernel<T, S, NT, MINB, false, true, PER><<<grid, NT, G::smem_bytes, h->stream>>>(inF, inA, outF, outA, h->kp, h->march_nseg);
+        return launch_chained(march_pair_kernel<T, S, NT, MINB, false, true, PER>, grid, NT, G::smem_bytes, h->stream, inF, inA, outF, outA, h->kp, h->march_nseg);
     else
-        march_pair_kernel<T, S, NT, MINB, false, false, PER><<<grid, NT, G::smem_bytes, h->stream>>>(inF, inA, outF, outA, h->kp, h->march_nseg);
-    return cudaGetLastError();
+        return launch_chained(march_pair_kernel<T, S, NT, MINB, false, false, PER>, grid, NT, G::smem_bytes, h->stream, inF, inA, outF, outA, h->kp, h->march_nseg);
 }
 
 // Marching kernel variants: 0 = 64 threads at <= 128 registers (strips of
@@ -518,8 +538,9 @@ static cudaError_t launch_moments(hlbm_handle *h)
     const float *in = static_cast<const float *>(h->state[h->cur]);
     float *out = static_cast<float *>(h->state[h->cur ^ 1]);
     // one launch through the selected instantiation's pointer
-    void *args[] = {(void *)&in, (void *)&out, (void *)&h->kp, (void *)&h->march_nseg};
-    return cudaLaunchKernel(moment_kernel_ptr(h), grid, dim3(kMomNT), args, G::smem_bytes, h->stream);
+    auto kernel = reinterpret_cast<decltype(&march_moment_kernel<kMomNT, kMomMinB, false, true, true>)>(
+        const_cast<void *>(moment_kernel_ptr(h)));
+    return launch_chained(kernel, grid, dim3(kMomNT), G::smem_bytes, h->stream, in, out, h->kp, h->march_nseg);
 }
 
 // Level-n ghost rows of the wall sides, from the current state.
@@ -529,9 +550,9 @@ static cudaError_t launch_wall_ghosts(hlbm_handle *h)
         using T = typename decltype(ty)::t;
         using S = typename decltype(ty)::s;
         dim3 grid((std::max(h->kp.wall_p, h->kp.wall_q) + 127) / 128, 8);
-        wall_ghost_kernel<T, S><<<grid, 128, 0, h->stream>>>(pop_planes<T, S>(h, h->cur), aux_planes<T, S>(h, h->cur),
-                                                             h->kp);
-        return cudaGetLastError();
+        return launch_chained(wall_ghost_kernel<T, S>, grid, 128, 0, h->stream,
+                              (const typename S::raw *)pop_planes<T, S>(h, h->cur), (const T *)aux_planes<T, S>(h, h->cur),
+                              h->kp);
     });
 }
 
@@ -551,9 +572,20 @@ static cudaError_t launch_one_step(hlbm_handle *h)
             return march_dispatch<T, S, true>(h);
         });
     }
-    if (h->p.precision == HLBM_FP64) return launch_step<double, FullStore<double>, TX64, TY64, NT64>(h);
-    if (h->p.precision == HLBM_FP32_F16POP) return launch_step<float, HalfStore, 32, 32, 512>(h);
-    if (h->p.precision == HLBM_FP32_BF16POP) return launch_step<float, BF16Store, 32, 32, 512>(h);
+    if (h->p.precision == HLBM_FP64) {
+        // walls, or HLBM_MARCH=-1: the SMs' FP64 pipes bound the tile, so a
+        // grid is cut as finely as still gives every SM one tile.  Per step
+        // with two walls (us; the former tile, 32x8 with 256 threads, last):
+        //   2 x 100  8x8 30.3, 16x8 35.0, 16x16 49.9, 54.6;  128^2  41.1, 37.2, 53.1, 58.1;
+        //   200 x 333  113, 95.5, 88.8, 126;  1000 x 900  1159, 955, 890, 909
+        using S = FullStore<double>;
+        auto tiles = [&](int tx, int ty) { return (long long)((h->p.nx + tx - 1) / tx) * ((h->p.ny + ty - 1) / ty); };
+        if (tiles(8, 8) <= kSms) return launch_step<double, S, 8, 8, 192>(h);
+        if (tiles(16, 8) <= kSms) return launch_step<double, S, 16, 8, 256>(h);
+        return launch_step<double, S, 16, 16, 512>(h);
+    }
+    if (h->p.precision == HLBM_FP32_F16POP) return launch_step<float, HalfStore, 16, 16, 512>(h);
+    if (h->p.precision == HLBM_FP32_BF16POP) return launch_step<float, BF16Store, 16, 16, 512>(h);
     if (h->tma_ready) {
         switch (h->tma_variant) {
         case 1: return launch_tma<32, 16, 256>(h);
@@ -567,6 +599,7 @@ static cudaError_t launch_one_step(hlbm_handle *h)
     case 2: return launch_step<float, F32, 32, 8, 128>(h);
     case 3: return launch_step<float, F32, 64, 32, 512>(h);
     case 4: return launch_step<float, F32, 32, 32, 512>(h);
+    case 5: return launch_step<float, F32, 16, 16, 512>(h);
     default: return launch_step<float, F32, 32, 16, 256>(h);
     }
 }
@@ -789,7 +822,7 @@ int hlbm_create(const hlbm_params *params, void *stream, hlbm_handle **out)
         h->kp.wall_g = h->wall_g;
         h->kp.wall_p = params->nx + 4;
         h->kp.wall_q = params->ny + 4;
-        h->tile_variant = env_choice("HLBM_FP32_TILE", 4, 0, kNumFp32Tiles);
+        h->tile_variant = env_choice("HLBM_FP32_TILE", 5, 0, kNumFp32Tiles);
         *out = h;
         return HLBM_OK;
     }
@@ -803,7 +836,7 @@ int hlbm_create(const hlbm_params *params, void *stream, hlbm_handle **out)
         return HLBM_OK;
     }
     // FP64: the two-pass form at every size (1024^2 vortex 377 us per step
-    // against 764 on the marching kernel; Sod tube 400 x 4 19 us against 39
+    // against 764 on the marching kernel; Sod tube 400 x 4 13 us against 39
     // on the tiled kernel).  HLBM_MARCH=<k> picks a marching variant, -1 the
     // tiled kernel, as for the other precisions.
     if (two_pass) {

@@ -11,11 +11,12 @@
 // pitch is nx rounded up to 32 elements so that every row starts on a
 // 128-byte boundary.  rho and u of a level are the moments of F (collision
 // invariants, eqs. rhoalgo, ualgo) and theta follows from s and rho; only the
-// FP64 row-marching form also stores them, in four planes behind these
+// FP64 two-pass and row-marching forms also store them, in four planes behind these
 // (A_RHO .. A_TH), so that no step recomputes them.
 //
-// This file holds the tiled form of the step (FP64, and FP32 grids of up to
-// 768^2 cells) with the scalar cell arithmetic; hlbm_march.cuh holds the
+// This file holds the tiled form of the step (FP32 grids of up to 768^2
+// cells, and every grid with wall sides) with the scalar cell arithmetic;
+// hlbm_split.cuh holds the FP64 form in two passes, and hlbm_march.cuh the
 // row-marching form (the FP32 default on larger grids, the batched form's
 // marching shapes, and the moment-state form).
 //
@@ -60,6 +61,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "hlbm_tables64.h"
+
 namespace hlbm {
 
 // ---- index checks of the debug build (HLBM_DEBUG) --------------------------------
@@ -97,6 +100,22 @@ __device__ __forceinline__ bool dbg_range(long long v, long long n, int site)
 #define HLBM_CELL_OK(row, col, width, kp, site) true
 #define HLBM_RANGE_OK(v, n, site) true
 #endif
+
+// ---- steps that follow each other on a stream -------------------------------------
+// The step kernels are launched with programmatic stream serialisation: a
+// step's CTAs may be set up while the last CTAs of the step before still
+// run.  Every kernel launched that way reads and writes no memory that
+// another kernel writes before step_begin(), which waits until the kernel
+// before it has completed and its writes are visible.  step_next() lets the
+// next kernel's CTAs be set up once every CTA of this one has called it.  It
+// stands at a kernel's end: CTAs that wait for a whole step occupy an SM's
+// slots unevenly (march kernel at 1024^2, per step: 31.6 us without, 30.1 with
+// step_next() at the start, 28.9 at the end; at 800^2 26.8, 29.5, 25.2).
+__device__ __forceinline__ void step_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void step_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 constexpr int NPLANE = 13;
 constexpr int P_S = 9, P_AXX = 10, P_AXY = 11, P_AYY = 12;
@@ -288,6 +307,73 @@ __device__ __forceinline__ float ex2_approx(float x)
     return r;
 }
 
+// ---- FP64 logarithm and exponential ------------------------------------------
+// log x and exp x by the table-driven methods of P. T. P. Tang (ACM TOMS 16,
+// 1990, and 15, 1989): 12 and 12 FP64 operations where CUDA's functions take
+// 32 and 17 dependent ones on this GPU (2030 and 1109 cycles at the 64 cycles
+// a warp's FP64 instruction takes).
+//   log: x = 2^k m, r = m c - 1 with c near 1 / m from the table, so |r| <=
+//   2^-7 and log x = k log 2 - log c + log(1 + r); the interval is centred so
+//   that k = 0 and c = 1 around x = 1, where the relative error stays small.
+//   exp: x = (128 n + j) log 2 / 128 + r, |r| < 2^-8.5, exp x = 2^n 2^(j/128) e^r.
+// The truncated series leave 2^-59 and 2^-60 relative; against 64-bit mantissas
+// the largest errors found are 1.4 and 0.51 ulp (2 10^7 points per range, 64-bit
+// mantissas).  theta itself, whose exponent is rounded before the exponential,
+// is off by 3.1e-16 relative at most and 1.07e-16 rms for rho in 0.9 .. 1.1 and
+// theta in 0.15 .. 0.25, the same figures as with correctly rounded functions.  Operands outside the normal range take CUDA's functions.
+//
+// The tables are copied to shared memory at the start of a pass, so that a
+// lookup, which stands in the chain of dependent operations, is no trip to L2.
+struct Tables64 {
+    double2 log[128], exp[128];
+    double low[128];
+};
+__device__ __forceinline__ void load_tables64(Tables64 &t)
+{
+    for (int i = threadIdx.y * blockDim.x + threadIdx.x; i < 128; i += blockDim.x * blockDim.y) {
+        t.log[i] = __ldg(&kLogTable[i]);
+        t.exp[i] = __ldg(&kExpTable[i]);
+        t.low[i] = __ldg(&kLogLow[i]);
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ double log64(const Tables64 &tab, double x)
+{
+    const int hi = __double2hiint(x);
+    if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // not a positive normal number
+    const int i = (hi >> 13) & 127, up = i >= 53;
+    const int k = (hi >> 20) - 1023 + up;
+    const double m = __hiloint2double((hi & 0x000fffff) | (up ? 0x3fe00000 : 0x3ff00000), __double2loint(x));
+    const double2 c = tab.log[i];
+    const double r = fma(m, c.x, -1.0);
+    double q = fma(r, -1.0 / 8.0, 1.0 / 7.0);
+    q = fma(r, q, -1.0 / 6.0);
+    q = fma(r, q, 1.0 / 5.0);
+    q = fma(r, q, -1.0 / 4.0);
+    q = fma(r, q, 1.0 / 3.0);
+    q = fma(r, q, -1.0 / 2.0);
+    const double l = fma(r * r, q, r) + tab.low[i];
+    return (k == 0 ? c.y : fma((double)k, kLn2, c.y)) + l;
+}
+
+__device__ __forceinline__ double exp64(const Tables64 &tab, double x)
+{
+    if ((unsigned)(__double2hiint(x) & 0x7fffffff) >= 0x4082c000u) return exp(x);  // |x| >= 600 or NaN
+    const double magic = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the rounded integer
+    const double t = fma(x, k128OverLn2, magic);
+    const int n = __double2loint(t);
+    const double kd = t - magic;
+    const double r = fma(kd, -kLn2Over128Lo, fma(kd, -kLn2Over128Hi, x));
+    const double2 c = tab.exp[n & 127];
+    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    q = fma(r, q, 1.0 / 6.0);
+    q = fma(r, q, 0.5);
+    const double p = fma(r * r, q, r);  // e^r - 1
+    const double y = c.x + fma(c.x, p, c.y);
+    return __hiloint2double(__double2hiint(y) + ((n >> 7) << 20), __double2loint(y));
+}
+
 // ---- precision-dependent helpers -------------------------------------------
 template <typename T> struct Consts;
 
@@ -454,28 +540,21 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
     const long long P = kp.plane;
     const bool interior = x0 >= 3 && y0 >= 3 && x0 + TX + 3 <= kp.nx && y0 + TY + 3 <= kp.ny;
 
-    // phase 0 + 1 loads: s(n) on tile + 3 and F(n) on tile + 2 go to shared
-    // memory first, with all of a thread's loads in flight together
-    for (int c = threadIdx.x; c < N3; c += NT) {
-        const int ly = c / R3X, lx = c - ly * R3X;
-        const int gx = x0 - 3 + lx, gy = y0 - 3 + ly;
-        const int o = interior ? gy * pitch + gx : locate_w(gx, gy, kp, pitch);
-        sS[c] = o >= 0 ? (HLBM_CELL_OK(o / pitch, o % pitch, 1, kp, 10) ? __ldg(inA + A_S * P + o) : T(0))
-                       : (o > -kWallCode ? side.s_(-o - 1) : wall_val<T>(kp, -o - kWallCode, 9));
-    }
+    // phase 0 + 1 loads: F(n) on tile + 2, s(n) on tile + 3 and, where a
+    // thread has one phase-2 cell at most, its a1(n) (phi_mode 0), all in
+    // flight together: on a small grid a step is a chain of such trips
+    constexpr bool ONE = N1 <= NT;
+    T a1n[3] = {T(0), T(0), T(0)};
     {
         constexpr int ITER = (N2 + NT - 1) / NT;
         T f[ITER][9];
-        int oc[ITER];
 #pragma unroll
         for (int it = 0; it < ITER; it++) {
             const int c = threadIdx.x + it * NT;
-            oc[it] = 0;
             if (c < N2) {
                 const int ly = c / R2X, lx = c - ly * R2X;
                 const int gx = x0 - 2 + lx, gy = y0 - 2 + ly;
                 const int o = interior ? gy * pitch + gx : locate_w(gx, gy, kp, pitch);
-                oc[it] = o;
                 if (o >= 0) {
                     const bool ok = HLBM_CELL_OK(o / pitch, o % pitch, 1, kp, 11);
 #pragma unroll
@@ -489,6 +568,22 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
                 }
             }
         }
+        if (ONE && (int)threadIdx.x < N1 && kp.phi_mode == 0) {
+            const int ly = threadIdx.x / R1X, lx = threadIdx.x - ly * R1X;
+            const int gx = x0 - 1 + lx, gy = y0 - 1 + ly;
+            const int o = interior ? gy * pitch + gx : locate(gx, gy, kp, pitch);
+            if (o >= 0) {
+#pragma unroll
+                for (int k = 0; k < 3; k++) a1n[k] = __ldg(inA + (A_XX + k) * P + o);
+            }
+        }
+        for (int c = threadIdx.x; c < N3; c += NT) {
+            const int ly = c / R3X, lx = c - ly * R3X;
+            const int gx = x0 - 3 + lx, gy = y0 - 3 + ly;
+            const int o = interior ? gy * pitch + gx : locate_w(gx, gy, kp, pitch);
+            sS[c] = o >= 0 ? (HLBM_CELL_OK(o / pitch, o % pitch, 1, kp, 10) ? __ldg(inA + A_S * P + o) : T(0))
+                           : (o > -kWallCode ? side.s_(-o - 1) : wall_val<T>(kp, -o - kWallCode, 9));
+        }
 #pragma unroll
         for (int it = 0; it < ITER; it++) {
             const int c = threadIdx.x + it * NT;
@@ -497,7 +592,6 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
                 for (int i = 0; i < 9; i++) sF[i * N2 + c] = f[it][i];
             }
         }
-        (void)oc;
     }
     __syncthreads();
 
@@ -544,8 +638,8 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
         }
         // a1(n) of this cell (phi_mode 0): issued first so the loads overlap
         // the stencil arithmetic below
-        T axx = T(0), axy = T(0), ayy = T(0);
-        if (kp.phi_mode == 0) {
+        T axx = a1n[0], axy = a1n[1], ayy = a1n[2];
+        if (!ONE && kp.phi_mode == 0) {
             const int o = interior ? gy * pitch + gx : locate(gx, gy, kp, pitch);
             if (o >= 0) {
                 axx = __ldg(inA + A_XX * P + o); axy = __ldg(inA + A_XY * P + o); ayy = __ldg(inA + A_YY * P + o);
@@ -627,8 +721,13 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
         }
     }
 
-    // phase 3: psi, f^eq, a1 and the collision of the next step on the tile
-    for (int c = threadIdx.x; c < TX * TY; c += NT) {
+    // phase 3: psi, f^eq, a1 and the collision of the next step on the tile.
+    // The trip count is hidden from the compiler, so that a tile shape whose
+    // threads have one cell each gets the same instructions, and rounding, as
+    // the others.
+    int cells = TX * TY;
+    asm("" : "+r"(cells));
+    for (int c = threadIdx.x; c < cells; c += NT) {
         const int ly = c / TX, lx = c - ly * TX;
         const int gx = x0 + lx, gy = y0 + ly;
         if (gx >= kp.nx || gy >= kp.ny) continue;
@@ -695,7 +794,9 @@ fused_step_kernel(const typename S::raw *__restrict__ inF, const T *__restrict__
                   typename S::raw *__restrict__ outF, T *__restrict__ outA, const KParams kp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    step_begin();
     step_tile<T, S, TX, TY, NT>(inF, inA, outF, outA, kp, blockIdx.x * TX, blockIdx.y * TY, smem_raw);
+    step_next();
 }
 
 // ---- many cases in one persistent launch (FP32) -----------------------------------
@@ -769,6 +870,10 @@ template <typename T, typename S>
 __global__ void wall_ghost_kernel(const typename S::raw *__restrict__ inF, const T *__restrict__ inA,
                                   const KParams kp)
 {
+    constexpr bool W16 = sizeof(typename S::raw) == 2;
+    __shared__ Tables64 tab;
+    if (!W16) load_tables64(tab);
+    step_begin();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int layer = blockIdx.y;
     const bool xw = layer >= 4;
@@ -824,7 +929,12 @@ __global__ void wall_ghost_kernel(const typename S::raw *__restrict__ inF, const
     const size_t stride = (size_t)4 * kp.wall_p + (size_t)4 * kp.wall_q;
 #pragma unroll
     for (int q = 0; q < 9; q++) wg[q * stride + w] = f[q];
-    wg[9 * stride + w] = (T)(kp.cv * (log((double)c.th) - kp.gm1 * log((double)c.rho)));
+    // (16-bit populations keep CUDA's logarithm: a rounding that differs once
+    // in FP32 grows to their own quantisation error within a few steps)
+    const double lt = W16 ? log((double)c.th) : log64(tab, (double)c.th);
+    const double lr = W16 ? log((double)c.rho) : log64(tab, (double)c.rho);
+    wg[9 * stride + w] = (T)(kp.cv * (lt - kp.gm1 * lr));
+    step_next();
 }
 
 // ---- initialisation (Sec. 3.5: f^eq, a1^FD and psi of the input state) --------

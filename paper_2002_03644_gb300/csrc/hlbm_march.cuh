@@ -620,9 +620,11 @@ march_pair_kernel(const typename S::raw *__restrict__ inF, const T *__restrict__
                   typename S::raw *__restrict__ outF, T *__restrict__ outA, const KParams kp, const int nseg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    step_begin();
     const int ys = seg_start(blockIdx.y, nseg, kp.ny), ye = seg_start(blockIdx.y + 1, nseg, kp.ny);
     march_pair_segment<T, S, NT, SIG, PHI0, PER>(inF, inA, outF, outA, kp, blockIdx.x * PairGeom<T, NT>::W, ys, ye,
                                                  smem_raw);
+    step_next();
 }
 
 // FP64 row-marching form: the cache planes of a state whose level-n values
@@ -1096,8 +1098,10 @@ __global__ void __launch_bounds__(NT, MINB)
 march_moment_kernel(const float *__restrict__ in, float *__restrict__ out, const KParams kp, const int nseg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    step_begin();
     const int ys = seg_start(blockIdx.y, nseg, kp.ny), ye = seg_start(blockIdx.y + 1, nseg, kp.ny);
     moment_segment<NT, SIG, PHI0, PER>(in, out, kp, blockIdx.x * MomGeom<NT>::W, ys, ye, smem_raw);
+    step_next();
 }
 
 // Moment state from FP64 caller fields (the initialisation of Sec. 3.5): rho, u, s

@@ -22,7 +22,7 @@
 // instead of eight divisions.
 //
 // Measured on GB300, per step: 1024^2 vortex 377 us (764 on the marching
-// kernel), Sod tube 400 x 4 19 us (39 on the tiled kernel).  The FP64 pipe is
+// kernel), Sod tube 400 x 4 13 us (39 on the tiled kernel).  The FP64 pipe is
 // busy for 84 % of the level and the collide pass's cycles, which is what 19
 // cycles per warp instruction, the most that eight warps of dependent
 // multiply-adds reach, come to.
@@ -40,7 +40,6 @@
 #pragma once
 
 #include "hlbm_march.cuh"
-#include "hlbm_tables64.h"
 
 namespace hlbm {
 
@@ -72,72 +71,6 @@ __device__ __forceinline__ double rcp64(double b)
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
     const double e = fma(-b, y, 1.0);
     return fma(y, fma(e, e, e), y);
-}
-
-// log x and exp x by the table-driven methods of P. T. P. Tang (ACM TOMS 16,
-// 1990, and 15, 1989): 12 and 12 FP64 operations where CUDA's functions take
-// 32 and 17 dependent ones on this GPU (2030 and 1109 cycles at the 64 cycles
-// a warp's FP64 instruction takes).
-//   log: x = 2^k m, r = m c - 1 with c near 1 / m from the table, so |r| <=
-//   2^-7 and log x = k log 2 - log c + log(1 + r); the interval is centred so
-//   that k = 0 and c = 1 around x = 1, where the relative error stays small.
-//   exp: x = (128 n + j) log 2 / 128 + r, |r| < 2^-8.5, exp x = 2^n 2^(j/128) e^r.
-// The truncated series leave 2^-59 and 2^-60 relative; against 64-bit mantissas
-// the largest errors found are 1.4 and 0.51 ulp (2 10^7 points per range, 64-bit
-// mantissas).  theta itself, whose exponent is rounded before the exponential,
-// is off by 3.1e-16 relative at most and 1.07e-16 rms for rho in 0.9 .. 1.1 and
-// theta in 0.15 .. 0.25, the same figures as with correctly rounded functions.  Operands outside the normal range take CUDA's functions.
-//
-// The tables are copied to shared memory at the start of a pass, so that a
-// lookup, which stands in the chain of dependent operations, is no trip to L2.
-struct Tables64 {
-    double2 log[128], exp[128];
-    double low[128];
-};
-__device__ __forceinline__ void load_tables64(Tables64 &t)
-{
-    for (int i = threadIdx.y * blockDim.x + threadIdx.x; i < 128; i += blockDim.x * blockDim.y) {
-        t.log[i] = __ldg(&kLogTable[i]);
-        t.exp[i] = __ldg(&kExpTable[i]);
-        t.low[i] = __ldg(&kLogLow[i]);
-    }
-    __syncthreads();
-}
-
-__device__ __forceinline__ double log64(const Tables64 &tab, double x)
-{
-    const int hi = __double2hiint(x);
-    if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // not a positive normal number
-    const int i = (hi >> 13) & 127, up = i >= 53;
-    const int k = (hi >> 20) - 1023 + up;
-    const double m = __hiloint2double((hi & 0x000fffff) | (up ? 0x3fe00000 : 0x3ff00000), __double2loint(x));
-    const double2 c = tab.log[i];
-    const double r = fma(m, c.x, -1.0);
-    double q = fma(r, -1.0 / 8.0, 1.0 / 7.0);
-    q = fma(r, q, -1.0 / 6.0);
-    q = fma(r, q, 1.0 / 5.0);
-    q = fma(r, q, -1.0 / 4.0);
-    q = fma(r, q, 1.0 / 3.0);
-    q = fma(r, q, -1.0 / 2.0);
-    const double l = fma(r * r, q, r) + tab.low[i];
-    return (k == 0 ? c.y : fma((double)k, kLn2, c.y)) + l;
-}
-
-__device__ __forceinline__ double exp64(const Tables64 &tab, double x)
-{
-    if ((unsigned)(__double2hiint(x) & 0x7fffffff) >= 0x4082c000u) return exp(x);  // |x| >= 600 or NaN
-    const double magic = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are the rounded integer
-    const double t = fma(x, k128OverLn2, magic);
-    const int n = __double2loint(t);
-    const double kd = t - magic;
-    const double r = fma(kd, -kLn2Over128Lo, fma(kd, -kLn2Over128Hi, x));
-    const double2 c = tab.exp[n & 127];
-    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    q = fma(r, q, 1.0 / 6.0);
-    q = fma(r, q, 0.5);
-    const double p = fma(r * r, q, r);  // e^r - 1
-    const double y = c.x + fma(c.x, p, c.y);
-    return __hiloint2double(__double2hiint(y) + ((n >> 7) << 20), __double2loint(y));
 }
 
 // theta = rho^(gamma - 1) exp(s / c_v) (eq. Entropie expression)
@@ -220,6 +153,8 @@ split_level_kernel(const double *__restrict__ F, const double *__restrict__ A, d
 {
     __shared__ Tables64 tab;
     load_tables64(tab);
+    step_begin();
+    step_next();  // at the start: Sod tube 12.9 us per step against 14.1 at the end, 1024^2 alike
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= kp.nx || y >= kp.ny) return;
     const long long P = kp.plane;
@@ -345,6 +280,8 @@ split_collide_kernel(double *__restrict__ F, double *A, const SplitPlanes sp, co
 {
     __shared__ Tables64 tab;
     if (CANON) load_tables64(tab);
+    step_begin();
+    step_next();
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= kp.nx || y >= kp.ny) return;
     const long long P = kp.plane;
