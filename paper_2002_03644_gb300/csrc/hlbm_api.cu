@@ -946,8 +946,19 @@ int hlbm_init_fields(hlbm_handle *h, const double *rho, const double *ux, const 
     } else CK(with_types(h, [&](auto ty) {
            using T = typename decltype(ty)::t;
            using S = typename decltype(ty)::s;
-           init_kernel<T, S><<<cell_grid(h, blk), blk, 0, h->stream>>>(dev[0], dev[1], dev[2], dev[3], dev[4],
-                                                                       pop_planes<T, S>(h, 0), aux_planes<T, S>(h, 0), h->kp);
+           const T *f[4];
+           if constexpr (std::is_same<T, double>::value) {
+               for (int k = 0; k < 4; k++) f[k] = dev[k];
+           } else {
+               // planes 7 and 8 of the staging buffer: free here (staged host
+               // fields take planes 0 .. 6)
+               float *conv = reinterpret_cast<float *>(h->staging + 7 * n);
+               convert_fields_kernel<<<dim3((unsigned)std::min<size_t>((n + 255) / 256, 4 * kSms), 4), 256, 0, h->stream>>>(
+                   dev[0], dev[1], dev[2], dev[3], conv, (long long)n);
+               for (int k = 0; k < 4; k++) f[k] = conv + k * n;
+           }
+           init_kernel<T, S><<<cell_grid(h, blk), blk, 0, h->stream>>>(f[0], f[1], f[2], f[3], dev[4], pop_planes<T, S>(h, 0),
+                                                                       aux_planes<T, S>(h, 0), h->kp);
            return cudaGetLastError();
        }), "init_kernel");
     h->cur = 0;

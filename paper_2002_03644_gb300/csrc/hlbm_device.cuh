@@ -374,6 +374,37 @@ __device__ __forceinline__ double exp64(const Tables64 &tab, double x)
     return __hiloint2double(__double2hiint(y) + ((n >> 7) << 20), __double2loint(y));
 }
 
+// 1 / b: the hardware's approximation y0 (20 bits) and one step of the
+// third-order iteration y0 (1 + e + e^2), e = 1 - b y0 (Householder's method
+// for the reciprocal; the remaining error e^3 is below 2^-59), three
+// multiply-adds where the IEEE division takes about nine FP64 instructions.
+// The last operation rounds once, so the result is within 0.51 ulp.
+// Operands near the ends of the exponent range, zero, infinite or NaN take
+// the division.
+__device__ __forceinline__ double rcp64(double b)
+{
+    const unsigned ex = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
+    if (ex - 64u >= 1920u) return 1.0 / b;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = fma(-b, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// theta = rho^(gamma - 1) exp(s / c_v) (eq. Entropie expression)
+__device__ __forceinline__ double theta64(const Tables64 &tab, const KParams &kp, double rho, double s)
+{
+    return exp64(tab, fma(kp.gm1, log64(tab, rho), __dmul_rn(s, kp.inv_cv)));
+}
+
+// a / b from ib = rcp64(b): one correction, which leaves little more than the
+// final rounding
+__device__ __forceinline__ double div64(double a, double b, double ib)
+{
+    const double q = a * ib;
+    return fma(fma(-b, q, a), ib, q);
+}
+
 // ---- precision-dependent helpers -------------------------------------------
 template <typename T> struct Consts;
 
@@ -953,9 +984,25 @@ __device__ __forceinline__ float init_entropy(const KParams &kp, float rho, floa
 // arithmetic is in T as well: the FP32-arithmetic forms round the fields to
 // FP32 on load, as their step does with every level, and FP64 computes in
 // FP64 throughout.
+//
+// The fields are given in the arithmetic type: a conversion from FP64 takes
+// the FP64 pipe (19 cycles per warp and SM), and converting a cell's value
+// for itself and again for each of its neighbours, 20 conversions per cell,
+// was what bound the initialisation of the FP32 forms (790 us at 4096^2).
+// convert_fields_kernel converts each value once (154 + 257 us).
+__global__ void __launch_bounds__(256)
+convert_fields_kernel(const double *__restrict__ rho, const double *__restrict__ ux, const double *__restrict__ uy,
+                      const double *__restrict__ th, float *__restrict__ out, long long n)
+{
+    const double *src[4] = {rho, ux, uy, th};
+    const double *p = src[blockIdx.y];
+    float *q = out + (long long)blockIdx.y * n;
+    for (long long i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) q[i] = (float)p[i];
+}
+
 template <typename T, typename S>
-__global__ void init_kernel(const double *__restrict__ rho, const double *__restrict__ ux,
-                            const double *__restrict__ uy, const double *__restrict__ th,
+__global__ void init_kernel(const T *__restrict__ rho, const T *__restrict__ ux,
+                            const T *__restrict__ uy, const T *__restrict__ th,
                             const double *__restrict__ a1, typename S::raw *__restrict__ outF,
                             T *__restrict__ outA, const KParams kp)
 {
@@ -975,7 +1022,7 @@ __global__ void init_kernel(const double *__restrict__ rho, const double *__rest
             xx = xx < 0 ? -xx - 1 : 2 * kp.nx - 1 - xx;
         }
         const int o = locate(xx, yy, kp, kp.nx);
-        if (o >= 0) { r = (T)rho[o]; u = (T)ux[o]; v = (T)uy[o]; t = (T)th[o]; }
+        if (o >= 0) { r = rho[o]; u = ux[o]; v = uy[o]; t = th[o]; }
         else { const int s = -o - 1; r = (T)kp.d_rho[s]; u = (T)kp.d_ux[s]; v = (T)kp.d_uy[s]; t = (T)kp.d_th[s]; }
         if (ws >= 0) {
             const T tg = T(2) * (T)kp.d_th[ws] - t;
@@ -1028,6 +1075,9 @@ __global__ void macros_kernel(const typename S::raw *__restrict__ inF, const T *
                               double *ux, double *uy, double *th, double *s, double *a1, double *F,
                               const KParams kp)
 {
+    constexpr bool F64 = sizeof(T) == 8;
+    __shared__ Tables64 tab;
+    if (F64) load_tables64(tab);
     const int gx = blockIdx.x * blockDim.x + threadIdx.x;
     const int gy = blockIdx.y * blockDim.y + threadIdx.y;
     if (gx >= kp.nx || gy >= kp.ny) return;
@@ -1044,9 +1094,16 @@ __global__ void macros_kernel(const typename S::raw *__restrict__ inF, const T *
     moments(f, r, jx, jy);
     const T sv = inA[A_S * P + o];
     if (rho) rho[c] = (double)r;
-    if (ux) ux[c] = (double)(jx / r);
-    if (uy) uy[c] = (double)(jy / r);
-    if (th) th[c] = (double)cs.theta(r, sv);
+    if constexpr (F64) {
+        const double ir = rcp64(r);
+        if (ux) ux[c] = div64(jx, r, ir);
+        if (uy) uy[c] = div64(jy, r, ir);
+        if (th) th[c] = theta64(tab, kp, r, sv);
+    } else {
+        if (ux) ux[c] = (double)(jx / r);
+        if (uy) uy[c] = (double)(jy / r);
+        if (th) th[c] = (double)cs.theta(r, sv);
+    }
     if (s) s[c] = (double)sv;
     if (a1) {
         a1[c] = (double)inA[A_XX * P + o];

@@ -56,29 +56,6 @@ struct SplitPlanes {
 };
 constexpr int SPLIT_NPLANE = 8, SPLIT_NPLANE_CANON = 12;
 
-// 1 / b: the hardware's approximation y0 (20 bits) and one step of the
-// third-order iteration y0 (1 + e + e^2), e = 1 - b y0 (Householder's method
-// for the reciprocal; the remaining error e^3 is below 2^-59), three
-// multiply-adds where the IEEE division takes about nine FP64 instructions.
-// The last operation rounds once, so the result is within 0.51 ulp.
-// Operands near the ends of the exponent range, zero, infinite or NaN take
-// the division.
-__device__ __forceinline__ double rcp64(double b)
-{
-    const unsigned ex = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
-    if (ex - 64u >= 1920u) return 1.0 / b;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    const double e = fma(-b, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-
-// theta = rho^(gamma - 1) exp(s / c_v) (eq. Entropie expression)
-__device__ __forceinline__ double theta64(const Tables64 &tab, const KParams &kp, double rho, double s)
-{
-    return exp64(tab, fma(kp.gm1, log64(tab, rho), __dmul_rn(s, kp.inv_cv)));
-}
-
 // x > 0 and x < 0 of numbers, on the integer pipe (a comparison of doubles
 // takes the FP64 pipe like a multiply-add).
 __device__ __forceinline__ bool positive64(double x) { return __double_as_longlong(x) > 0; }
