@@ -45,13 +45,24 @@ BYTES_PER_CELL = {"fp32": 104, "fp64": 208, "fp16pop": 68, "bf16pop": 68, "momen
 # the FP64 marching kernel also reads and writes each cell's level rho, u_x,
 # u_y, theta (4 FP64 planes kept so that no step recomputes them)
 FP64_MARCH_BYTES_PER_CELL = 272
+# the two-pass FP64 form moves those, five planes from one pass to the other
+# (two closure defects, two slopes, a reciprocal) and reads s and the level's
+# rho, u_x, u_y, theta again in its second pass
+FP64_SPLIT_BYTES_PER_CELL = 272 + 10 * 8 + 5 * 8
+
+
+def fp64_split(precision):
+    """Whether a step is the two-pass FP64 form (the default without HLBM_MARCH)."""
+    return precision == "fp64" and "HLBM_MARCH" not in os.environ
 
 
 def bytes_per_cell(precision, cells):
     """Bytes one cell-update reads and writes in the fused-step kernel the
     library launches (kernel choice as in kernel_name)."""
+    if fp64_split(precision):
+        return FP64_SPLIT_BYTES_PER_CELL
     if precision == "fp64":
-        march = int(os.environ.get("HLBM_MARCH", "-1" if cells <= 768 * 768 else "0"))
+        march = int(os.environ["HLBM_MARCH"])
         if 0 <= march < 4:
             return FP64_MARCH_BYTES_PER_CELL
     return BYTES_PER_CELL[precision]
@@ -234,7 +245,12 @@ def kernel_name(precision, cells, sigma=0.0, phi_mode=0, periodic=False):
     row-marching kernel on grids of more than 768^2 cells unless
     HLBM_MARCH=-1 (then the tiled kernels, chosen for FP32 by HLBM_FP32_TMA /
     HLBM_FP32_TILE), the tiled kernel on small grids unless HLBM_MARCH
-    selects a marching variant."""
+    selects a marching variant; FP64 runs two passes unless HLBM_MARCH is
+    set."""
+    if fp64_split(precision):
+        b = lambda v: str(bool(v)).lower()
+        return "split_level_kernel<%s,%s,false> + split_collide_kernel<%s,false,%s>" % (
+            b(sigma > 0), b(phi_mode == 0), b(sigma > 0), b(cells <= 768 * 768))
     if precision == "moments":
         return "march_moment_kernel<64,8,%s,%s%s>" % (str(sigma > 0).lower(), str(phi_mode == 0).lower(),
                                                       ",true" if periodic else "")
@@ -249,17 +265,17 @@ def kernel_name(precision, cells, sigma=0.0, phi_mode=0, periodic=False):
                                                         1 if f64 else minb, str(sigma > 0).lower(),
                                                         str(phi_mode == 0).lower(), per)
     if precision == "fp64":
-        return "fused_step_kernel<double,FullStore<double>,32,8,256>"
+        return "fused_step_kernel<double,FullStore<double>,16,16,512>"
     if precision in ("fp16pop", "bf16pop"):
         st = "HalfStore" if precision == "fp16pop" else "BF16Store"
-        return f"fused_step_kernel<float,{st},32,32,512>"
+        return f"fused_step_kernel<float,{st},16,16,512>"
     tma = int(os.environ.get("HLBM_FP32_TMA", "0" if cells > 2048 * 2048 else "-1"))
     if tma >= 0:
         return ["fused_step_tma_kernel<32,16,512>", "fused_step_tma_kernel<32,16,256>",
                 "fused_step_tma_kernel<64,16,512>", "fused_step_tma_kernel<32,32,512>"][tma]
-    tile = int(os.environ.get("HLBM_FP32_TILE", "4"))
+    tile = int(os.environ.get("HLBM_FP32_TILE", "5"))
     return "fused_step_kernel<float,FullStore<float>,%s>" % ["32,16,256", "64,16,256", "32,8,128", "64,32,512",
-                                                             "32,32,512"][tile]
+                                                             "32,32,512", "16,16,512"][tile]
 
 
 FP64_NOMINAL_TFLOPS = 1.25
@@ -520,7 +536,7 @@ def run_ours(args):
         "data": "synthetic", "config": dict(describe(case, args.precision), parallelism=f"replicas{ws}",
                                             back_to_back_mlups=b2b),
         "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "clocks": clk.summary(),
-        "gpu_launches": args.steps,
+        "gpu_launches": args.steps * (2 if fp64_split(args.precision) else 1),
     }
     if batched is not None:
         line["batched"] = batched

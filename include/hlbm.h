@@ -137,10 +137,12 @@ typedef struct hlbm_handle hlbm_handle;
  * ping-pong state (13 planes per copy: 9 post-collision populations, s and
  * a1_xx, a1_xy, a1_yy; rows padded to a multiple of 32 elements, the pad
  * columns filled with NaN and never written) and FP64 staging buffers.  In
- * HLBM_FP64 on the row-marching kernel (grids above 768^2 without wall
- * sides) each copy has 4 more planes, each cell's rho, u_x, u_y, theta of
- * the level it holds (derived state: hlbm_init_fields computes them, each
- * step stores them for the next, checkpoints carry them).  The
+ * HLBM_FP64 without wall sides each copy has 4 more planes, each cell's rho,
+ * u_x, u_y, theta of the level it holds (derived state: hlbm_init_fields
+ * computes them, each step stores them for the next; checkpoints carry them
+ * on grids above 768^2 cells and derive them again on smaller ones), and
+ * the staging buffer 12 more planes for what the step's two passes hand to
+ * each other.  The
  * parameters are checked before any CUDA call: HLBM_ERR_ARG for grids
  * outside 1 .. 2^28 cells or values outside the ranges above (a periodic
  * side without a periodic partner included), HLBM_ERR_UNSUPPORTED for an
@@ -189,12 +191,12 @@ int hlbm_diagnostics(hlbm_handle *h, double out[8]);
 /* Checkpoint: the size of the state blob, and a byte-exact copy of the state
  * and step counter into / from host memory: a header, then the state's
  * planes (13 for the population forms, 7 for HLBM_FP32_MOMENTS, 17 for
- * HLBM_FP64 on the row-marching kernel: the 13 and the 4 planes of level-n
- * rho, u_x, u_y, theta).  A run resumed from a blob continues bitwise as the
+ * HLBM_FP64 on grids above 768^2 cells without wall sides: the 13 and the 4
+ * planes of level-n rho, u_x, u_y, theta).  A run resumed from a blob continues bitwise as the
  * run that wrote it.  set_state checks sizes, precision and a header; it
  * returns HLBM_ERR_STATE on any mismatch.  In FP64 it takes a blob of 13
  * or 17 planes whatever kernel the handle runs: a 13-plane blob set on a
- * marching handle has its 4 planes derived from F and s (the first step
+ * handle whose own blobs have 17 has its 4 planes derived from F and s (the first step
  * then agrees with the run that wrote it to rounding). */
 int hlbm_state_bytes(const hlbm_handle *h, size_t *bytes);
 int hlbm_get_state(hlbm_handle *h, void *buf, size_t bytes);
@@ -360,15 +362,15 @@ int hlbm_selftest_wait(void *stream, long long budget_cycles, int arrive);
 /* ---- index checks of the debug build ---------------------------------------
  * A debugging aid, not a method of the paper.  The library built with
  * HLBM_DEBUG (libhlbm_debug.so, see paper_2002_03644_gb300/build.py) checks
- * in the marching, moment-state and tiled step kernels the cell of every
- * global load and store against the grid (the partner column of 2-element
+ * in the marching, moment-state, tiled and two-pass step kernels the cell of
+ * every global load (in the two-pass kernels: of every cell and pull) and store against the grid (the partner column of 2-element
  * accesses too) and the ring slots of the marching kernel against the ring
  * depths.  A failed check skips its access (a load reads zero) and the first
  * one is recorded; no kernel traps.  This call waits for the whole device,
  * then reads and clears the record: *site = 0 when every check passed, else
  * the site (1-3 marching loads of F, s, a1; 4 marching store; 5 ring slot; 6
  * phase-2 pair; 10-12 tiled loads of s, F and tiled store; 21, 22 moment
- * loads; 24 moment store) with two values of the failed check in *a, *b (row
+ * loads; 24 moment store; 31, 32 two-pass FP64 kernels) with two values of the failed check in *a, *b (row
  * and column, or the value and its bound).  Any pointer may be NULL.  The
  * release build returns HLBM_ERR_UNSUPPORTED. */
 int hlbm_debug_check(long long *site, long long *a, long long *b);
