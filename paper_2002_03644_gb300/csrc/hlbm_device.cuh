@@ -111,6 +111,13 @@ __device__ __forceinline__ bool dbg_range(long long v, long long n, int site)
 // stands at a kernel's end: CTAs that wait for a whole step occupy an SM's
 // slots unevenly (march kernel at 1024^2, per step: 31.6 us without, 30.1 with
 // step_next() at the start, 28.9 at the end; at 800^2 26.8, 29.5, 25.2).
+//
+// The state that such a kernel reads is written by the kernel before it, while
+// its own CTAs are already there: it is not read-only for the kernel's life.
+// Its pointers carry no __restrict__ and no load of it is an __ldg, so that
+// the loads are ordinary ones, which the wait orders (its memory clobber does
+// not order read-only loads).  The outputs keep __restrict__, which is what
+// lets the compiler move these loads across the stores of the cells before.
 __device__ __forceinline__ void step_begin()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -552,7 +559,7 @@ __device__ __forceinline__ T gamma_defect(T rho, T ua, T th)
 // One tile of one time step of Algorithm 1 (all threads of the CTA take part;
 // the caller separates consecutive tiles with a barrier).
 template <typename T, typename S, int TX, int TY, int NT>
-__device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ inF, const T *__restrict__ inA,
+__device__ __forceinline__ void step_tile(const typename S::raw *inF, const T *inA,
                                           typename S::raw *__restrict__ outF, T *__restrict__ outA,
                                           const KParams &kp, const int x0, const int y0, unsigned char *smem_raw)
 {
@@ -605,14 +612,14 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
             const int o = interior ? gy * pitch + gx : locate(gx, gy, kp, pitch);
             if (o >= 0) {
 #pragma unroll
-                for (int k = 0; k < 3; k++) a1n[k] = __ldg(inA + (A_XX + k) * P + o);
+                for (int k = 0; k < 3; k++) a1n[k] = inA[(A_XX + k) * P + o];
             }
         }
         for (int c = threadIdx.x; c < N3; c += NT) {
             const int ly = c / R3X, lx = c - ly * R3X;
             const int gx = x0 - 3 + lx, gy = y0 - 3 + ly;
             const int o = interior ? gy * pitch + gx : locate_w(gx, gy, kp, pitch);
-            sS[c] = o >= 0 ? (HLBM_CELL_OK(o / pitch, o % pitch, 1, kp, 10) ? __ldg(inA + A_S * P + o) : T(0))
+            sS[c] = o >= 0 ? (HLBM_CELL_OK(o / pitch, o % pitch, 1, kp, 10) ? inA[A_S * P + o] : T(0))
                            : (o > -kWallCode ? side.s_(-o - 1) : wall_val<T>(kp, -o - kWallCode, 9));
         }
 #pragma unroll
@@ -673,7 +680,7 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
         if (!ONE && kp.phi_mode == 0) {
             const int o = interior ? gy * pitch + gx : locate(gx, gy, kp, pitch);
             if (o >= 0) {
-                axx = __ldg(inA + A_XX * P + o); axy = __ldg(inA + A_XY * P + o); ayy = __ldg(inA + A_YY * P + o);
+                axx = inA[A_XX * P + o]; axy = inA[A_XY * P + o]; ayy = inA[A_YY * P + o];
             }
         }
         // entropy update from level-n fields (eq sequaalgo)
@@ -821,7 +828,7 @@ __device__ __forceinline__ void step_tile(const typename S::raw *__restrict__ in
 // One case: one CTA per tile.
 template <typename T, typename S, int TX, int TY, int NT>
 __global__ void __launch_bounds__(NT)
-fused_step_kernel(const typename S::raw *__restrict__ inF, const T *__restrict__ inA,
+fused_step_kernel(const typename S::raw *inF, const T *inA,
                   typename S::raw *__restrict__ outF, T *__restrict__ outA, const KParams kp)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -898,8 +905,7 @@ __device__ __forceinline__ void wall_reflect(const Side<T> &side, int ws, WallCe
 }
 
 template <typename T, typename S>
-__global__ void wall_ghost_kernel(const typename S::raw *__restrict__ inF, const T *__restrict__ inA,
-                                  const KParams kp)
+__global__ void wall_ghost_kernel(const typename S::raw *inF, const T *inA, const KParams kp)
 {
     constexpr bool W16 = sizeof(typename S::raw) == 2;
     __shared__ Tables64 tab;

@@ -189,8 +189,7 @@ struct PairGeom {
 // case; all NT threads of the CTA take part (the caller separates
 // consecutive segments with a barrier).
 template <typename T, typename S, int NT, bool SIG, bool PHI0, bool PER>
-__device__ __forceinline__ void march_pair_segment(const typename S::raw *__restrict__ inF,
-                                                   const T *__restrict__ inA, typename S::raw *__restrict__ outF,
+__device__ __forceinline__ void march_pair_segment(const typename S::raw *inF, const T *inA, typename S::raw *__restrict__ outF,
                                                    T *__restrict__ outA, const KParams &kp, const int x0,
                                                    const int ys, const int ye, unsigned char *smem_raw)
 {
@@ -616,7 +615,7 @@ __device__ __forceinline__ void march_pair_segment(const typename S::raw *__rest
 // out).
 template <typename T, typename S, int NT, int MINB, bool SIG, bool PHI0, bool PER = false>
 __global__ void __launch_bounds__(NT, MINB)
-march_pair_kernel(const typename S::raw *__restrict__ inF, const T *__restrict__ inA,
+march_pair_kernel(const typename S::raw *inF, const T *inA,
                   typename S::raw *__restrict__ outF, T *__restrict__ outA, const KParams kp, const int nseg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -732,7 +731,7 @@ struct MomGeom {
 };
 
 template <int NT, bool SIG, bool PHI0, bool PER>
-__device__ __forceinline__ void moment_segment(const float *__restrict__ in, float *__restrict__ out,
+__device__ __forceinline__ void moment_segment(const float *in, float *__restrict__ out,
                                                const KParams &kp, const int x0, const int ys, const int ye,
                                                unsigned char *smem_raw)
 {
@@ -1095,7 +1094,7 @@ __device__ __forceinline__ void moment_segment(const float *__restrict__ in, flo
 
 template <int NT, int MINB, bool SIG, bool PHI0, bool PER = false>
 __global__ void __launch_bounds__(NT, MINB)
-march_moment_kernel(const float *__restrict__ in, float *__restrict__ out, const KParams kp, const int nseg)
+march_moment_kernel(const float *in, float *__restrict__ out, const KParams kp, const int nseg)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     step_begin();

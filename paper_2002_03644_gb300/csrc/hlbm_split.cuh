@@ -117,7 +117,7 @@ __device__ __forceinline__ Cross cross_of(int x, int y, const KParams &kp)
 // A plane's value at an offset, or a Dirichlet side's constant (DIR: some
 // side is a Dirichlet side).
 template <bool DIR>
-__device__ __forceinline__ double plane_at(const double *__restrict__ p, int o, const double *side)
+__device__ __forceinline__ double plane_at(const double *p, int o, const double *side)
 {
     if (DIR && o < 0) return side[-o - 1];
     return p[o];
@@ -125,7 +125,7 @@ __device__ __forceinline__ double plane_at(const double *__restrict__ p, int o, 
 
 template <bool SIG, bool PHI0, bool DIR>
 __global__ void __launch_bounds__(256)
-split_level_kernel(const double *__restrict__ F, const double *__restrict__ A, double *__restrict__ outA,
+split_level_kernel(const double *F, const double *A, double *__restrict__ outA,
                    const SplitPlanes sp, const KParams kp)
 {
     __shared__ Tables64 tab;
@@ -241,7 +241,7 @@ __device__ __forceinline__ void populations64(double rho, double ux, double uy, 
 
 // The two limited slopes of s at a cell.
 template <bool DIR>
-__device__ __forceinline__ void slopes64(const double *__restrict__ ps, int o, const Cross &c, const KParams &kp,
+__device__ __forceinline__ void slopes64(const double *ps, int o, const Cross &c, const KParams &kp,
                                          const SplitPlanes &sp)
 {
     const double s0 = ps[o];
