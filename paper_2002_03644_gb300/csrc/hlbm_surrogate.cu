@@ -1382,6 +1382,11 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
         }
         cp_async_wait0();
         tell(q);
+        // A CTA that gives up leaves no copy under way into shared memory that
+        // is the next CTA's: the boxes of the last rows are waited for here.
+        // (Otherwise the MMAs have long waited for them.)
+        for (int e = q > SLOTS ? q - SLOTS : 0; e < q; e++) mbar_wait(bar(G::BAR_FULL + e % SLOTS), (e / SLOTS) & 1);
+        __syncwarp();
     } else if (warp == TC_MMA_WARP) {
         if (lane == 0) {
             // ---- the MMAs of a tile whose input rows i-1, i, i+1 sit in slots
@@ -1410,7 +1415,8 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                 }
             };
             int q0 = 0, i = t0 % H;  // the tile's first row
-            for (int k = 0; k < my_tiles; k++) {
+            int k = 0;
+            for (; k < my_tiles; k++) {
                 if (!count_wait(ready_s, k)) break;
                 tc_fence_after();
                 if (flip) issue(tmem + (k & 1) * NOUT, q0, true);
@@ -1419,6 +1425,9 @@ conv_tc_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__rest
                 q0 += i == H - 1 ? 3 : 1;
                 i = i == H - 1 ? 0 : i + 1;
             }
+            // nor an MMA that reads shared memory or writes TMEM after both are
+            // given back, when the warps that read the accumulators gave up
+            for (int e = k > 2 ? k - 2 : 0; e < k; e++) mbar_wait(bar(G::BAR_ACC + (e & 1)), (e >> 1) & 1);
         }
         __syncwarp();
     } else if (warp == TC_READY_WARP) {
