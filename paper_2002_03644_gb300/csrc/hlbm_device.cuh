@@ -386,12 +386,16 @@ __device__ __forceinline__ double exp64(const Tables64 &tab, double x)
 // for the reciprocal; the remaining error e^3 is below 2^-59), three
 // multiply-adds where the IEEE division takes about nine FP64 instructions.
 // The last operation rounds once, so the result is within 0.51 ulp.
-// Operands near the ends of the exponent range, zero, infinite or NaN take
-// the division.
+// Only for b with rcp64_ok(): not near the ends of the exponent range, zero,
+// infinite or NaN.  Other quotients are divisions and never products with a
+// reciprocal, which would be infinite for a subnormal b whose quotient is
+// finite (0 / 5e-309 in the slope of an entropy that fades out to 0).
+__device__ __forceinline__ bool rcp64_ok(double b)
+{
+    return (((unsigned)__double2hiint(b) >> 20) & 0x7ffu) - 64u < 1920u;
+}
 __device__ __forceinline__ double rcp64(double b)
 {
-    const unsigned ex = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
-    if (ex - 64u >= 1920u) return 1.0 / b;
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
     const double e = fma(-b, y, 1.0);
@@ -404,12 +408,21 @@ __device__ __forceinline__ double theta64(const Tables64 &tab, const KParams &kp
     return exp64(tab, fma(kp.gm1, log64(tab, rho), __dmul_rn(s, kp.inv_cv)));
 }
 
-// a / b from ib = rcp64(b): one correction, which leaves little more than the
-// final rounding
-__device__ __forceinline__ double div64(double a, double b, double ib)
+// a / b by the reciprocal
+__device__ __forceinline__ double quot64(double a, double b) { return rcp64_ok(b) ? __dmul_rn(a, rcp64(b)) : a / b; }
+
+// x = a / b and y = c / b, with one correction of the product with the
+// reciprocal, which leaves little more than the final rounding
+__device__ __forceinline__ void div64(double a, double c, double b, double &x, double &y)
 {
-    const double q = a * ib;
-    return fma(fma(-b, q, a), ib, q);
+    if (!rcp64_ok(b)) {
+        x = a / b;
+        y = c / b;
+        return;
+    }
+    const double ib = rcp64(b), p = a * ib, q = c * ib;
+    x = fma(fma(-b, p, a), ib, p);
+    y = fma(fma(-b, q, c), ib, q);
 }
 
 // ---- precision-dependent helpers -------------------------------------------
@@ -1101,9 +1114,10 @@ __global__ void macros_kernel(const typename S::raw *__restrict__ inF, const T *
     const T sv = inA[A_S * P + o];
     if (rho) rho[c] = (double)r;
     if constexpr (F64) {
-        const double ir = rcp64(r);
-        if (ux) ux[c] = div64(jx, r, ir);
-        if (uy) uy[c] = div64(jy, r, ir);
+        double u, v;
+        div64(jx, jy, r, u, v);
+        if (ux) ux[c] = u;
+        if (uy) uy[c] = v;
         if (th) th[c] = theta64(tab, kp, r, sv);
     } else {
         if (ux) ux[c] = (double)(jx / r);

@@ -47,7 +47,7 @@ namespace hlbm {
 // pass to the next level pass), [ny][pitch] each; sigma > 0 alone needs the
 // second moments.
 struct SplitPlanes {
-    double *dx, *dy, *inv;     // limited slopes of s, 1 / (2 mu + p): collide pass -> next level pass
+    double *dx, *dy, *mp;      // limited slopes of s, mu / (2 mu + p): collide pass -> next level pass
     double *gx, *gy;           // Gamma_x, Gamma_y of level n+1: level pass -> collide pass
     double *mxx, *myy, *mxy;   // second moments of the pulled populations: level pass -> collide pass
     double *rho, *ux, *uy, *th;  // level n+1: level pass -> collide pass (CANON: not the state's own cache planes)
@@ -82,13 +82,40 @@ __device__ __forceinline__ void moments64(const double f[9], double &rho, double
 __device__ __forceinline__ double va_slope64(double a, double b)
 {
     const double ab = a * b;
-    return positive64(ab) ? ab * (a + b) * rcp64(fma(a, a, b * b)) : 0.0;
+    return positive64(ab) ? quot64(ab * (a + b), fma(a, a, b * b)) : 0.0;
 }
 
 // p and 2 mu + p, rounded operation by operation: the collide pass and
 // split_prepare_kernel give the same bits, so a resumed run continues bitwise.
 __device__ __forceinline__ double pressure64(double rho, double th) { return __dmul_rn(__dmul_rn(rho, th), 1.0 / 3.0); }
-__device__ __forceinline__ double inv_two_mu_p(double two_mu, double p) { return rcp64(__dadd_rn(two_mu, p)); }
+
+// omega = (2 mu - p) / (2 mu + p) (eq. streamalgo) and mu / (2 mu + p), the
+// factor of the Phi of the next level (eq. viscous heat discret).
+__device__ __forceinline__ void relaxation64(double two_mu, double mu, double p, double &omega, double &mp)
+{
+    const double b = __dadd_rn(two_mu, p);
+    if (rcp64_ok(b)) {
+        const double ib = rcp64(b);
+        omega = __dmul_rn(two_mu - p, ib);
+        mp = __dmul_rn(mu, ib);
+    } else {
+        omega = (two_mu - p) / b;
+        mp = mu / b;
+    }
+}
+
+// u = j / rho (eq. ualgo)
+__device__ __forceinline__ void velocity64(double jx, double jy, double rho, double &ux, double &uy)
+{
+    if (rcp64_ok(rho)) {
+        const double ir = rcp64(rho);
+        ux = __dmul_rn(jx, ir);
+        uy = __dmul_rn(jy, ir);
+    } else {
+        ux = jx / rho;
+        uy = jy / rho;
+    }
+}
 
 // rho, u and theta of a cell from the stored F and s.  The sums are rounded
 // one by one (never fused with the products that made f), so that values
@@ -98,9 +125,7 @@ __device__ __forceinline__ void canon_macros64(const Tables64 &tab, const double
 {
     double jx, jy;
     moments64(f, rho, jx, jy);
-    const double ir = rcp64(rho);
-    ux = __dmul_rn(jx, ir);
-    uy = __dmul_rn(jy, ir);
+    velocity64(jx, jy, rho, ux, uy);
     th = theta64(tab, kp, rho, s);
 }
 
@@ -174,16 +199,16 @@ split_level_kernel(const double *F, const double *A, double *__restrict__ outA,
     double phi;
     if (PHI0) {
         const double a_xx = A[A_XX * P + o], a_xy = A[A_XY * P + o], a_yy = A[A_YY * P + o];
-        phi = -(kp.mu * sp.inv[o]) * (a_xx * dxux + a_xy * (dyux + dxuy) + a_yy * dyuy);
+        phi = -sp.mp[o] * (a_xx * dxux + a_xy * (dyux + dxuy) + a_yy * dyuy);
     } else {
         const double d1 = dxux - dyuy, d2 = dyux + dxuy;
         phi = sp.quarter_mu * (d1 * d1 + d2 * d2);
     }
-    const double s = fma(fma(kp.lambda, lap, phi), rcp64(rho0 * th0), s0 - ad);
-    double rho, jx, jy;
+    const double rt = rho0 * th0, heat = fma(kp.lambda, lap, phi);
+    const double s = rcp64_ok(rt) ? fma(heat, rcp64(rt), s0 - ad) : (s0 - ad) + heat / rt;
+    double rho, jx, jy, ux, uy;
     moments64(f, rho, jx, jy);
-    const double ir = rcp64(rho);
-    const double ux = jx * ir, uy = jy * ir;
+    velocity64(jx, jy, rho, ux, uy);
     const double th = theta64(tab, kp, rho, s);
     outA[A_S * P + o] = s;
     sp.rho[o] = rho;
@@ -296,9 +321,10 @@ split_collide_kernel(double *__restrict__ F, double *A, const SplitPlanes sp, co
     } else {
         axx = fdxx; ayy = -fdxx; axy = fdxy;
     }
-    const double inv = inv_two_mu_p(sp.two_mu, p);
+    double omega, mp;
+    relaxation64(sp.two_mu, kp.mu, p, omega, mp);
     double f[9];
-    populations64(rho, ux, uy, th, axx, axy, ayy, ex, ey, (sp.two_mu - p) * inv, f);
+    populations64(rho, ux, uy, th, axx, axy, ayy, ex, ey, omega, f);
 #pragma unroll
     for (int i = 0; i < 9; i++) F[i * P + o] = f[i];
     A[A_XX * P + o] = axx;
@@ -311,10 +337,9 @@ split_collide_kernel(double *__restrict__ F, double *A, const SplitPlanes sp, co
         A[A_UX * P + o] = u;
         A[A_UY * P + o] = v;
         A[A_TH * P + o] = t;
-        sp.inv[o] = inv_two_mu_p(sp.two_mu, pressure64(r, t));
-    } else {
-        sp.inv[o] = inv;
+        relaxation64(sp.two_mu, kp.mu, pressure64(r, t), omega, mp);
     }
+    sp.mp[o] = mp;
     slopes64<DIR>(A + A_S * P, o, c, kp, sp);
 }
 
@@ -345,7 +370,9 @@ split_prepare_kernel(const double *__restrict__ F, double *A, const SplitPlanes 
         r = A[A_RHO * P + o];
         t = A[A_TH * P + o];
     }
-    sp.inv[o] = inv_two_mu_p(sp.two_mu, pressure64(r, t));
+    double omega, mp;
+    relaxation64(sp.two_mu, kp.mu, pressure64(r, t), omega, mp);
+    sp.mp[o] = mp;
     slopes64<DIR>(A + A_S * P, o, cross_of(x, y, kp), kp, sp);
 }
 
