@@ -56,13 +56,16 @@ struct SplitPlanes {
 };
 constexpr int SPLIT_NPLANE = 8, SPLIT_NPLANE_CANON = 12;
 
-// x > 0 and x < 0 of numbers, on the integer pipe (a comparison of doubles
-// takes the FP64 pipe like a multiply-add).
-__device__ __forceinline__ bool positive64(double x) { return __double_as_longlong(x) > 0; }
+// x > 0 and x < 0, false for NaN as the comparisons are, on the integer pipe (a
+// comparison of doubles takes the FP64 pipe like a multiply-add): the bits of
+// the smallest subnormal to infinity, and the same with the sign.
+__device__ __forceinline__ bool positive64(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) - 1 < 0x7ff0000000000000ull;
+}
 __device__ __forceinline__ bool negative64(double x)
 {
-    const long long b = __double_as_longlong(x);
-    return b < 0 && b != (long long)0x8000000000000000ull;  // not -0
+    return (unsigned long long)__double_as_longlong(x) - 0x8000000000000001ull < 0x7ff0000000000000ull;
 }
 
 // rho and momentum of nine populations (moments(), every operation rounded).
