@@ -363,14 +363,15 @@ int hlbm_selftest_wait(void *stream, long long budget_cycles, int arrive);
  * A debugging aid, not a method of the paper.  The library built with
  * HLBM_DEBUG (libhlbm_debug.so, see paper_2002_03644_gb300/build.py) checks
  * in the marching, moment-state, tiled and two-pass step kernels the cell of
- * every global load (in the two-pass kernels: of every cell and pull) and store against the grid (the partner column of 2-element
+ * every global load and store against the grid (the partner column of 2-element
  * accesses too) and the ring slots of the marching kernel against the ring
  * depths.  A failed check skips its access (a load reads zero) and the first
  * one is recorded; no kernel traps.  This call waits for the whole device,
  * then reads and clears the record: *site = 0 when every check passed, else
  * the site (1-3 marching loads of F, s, a1; 4 marching store; 5 ring slot; 6
  * phase-2 pair; 10-12 tiled loads of s, F and tiled store; 21, 22 moment
- * loads; 24 moment store; 31, 32 two-pass FP64 kernels) with two values of the failed check in *a, *b (row
+ * loads; 24 moment store; 31, 32 the two passes of the FP64 step, 33 what
+ * prepares them) with two values of the failed check in *a, *b (row
  * and column, or the value and its bound).  Any pointer may be NULL.  The
  * release build returns HLBM_ERR_UNSUPPORTED. */
 int hlbm_debug_check(long long *site, long long *a, long long *b);

@@ -142,13 +142,14 @@ __device__ __forceinline__ Cross cross_of(int x, int y, const KParams &kp)
     return Cross{join_map(y, xw, kp.pitch), join_map(y, xe, kp.pitch), join_map(ys, x, kp.pitch), join_map(yn, x, kp.pitch)};
 }
 
-// A plane's value at an offset, or a Dirichlet side's constant (DIR: some
-// side is a Dirichlet side).
-template <bool DIR>
-__device__ __forceinline__ double plane_at(const double *p, int o, const double *side)
+// A plane's value at a neighbour's offset, or a Dirichlet side's constant
+// (DIR: some side is a Dirichlet side).  Every read of another cell goes
+// through here, where the debug build checks it.
+template <bool DIR, int SITE>
+__device__ __forceinline__ double plane_at(const double *p, int o, const double *side, const KParams &kp)
 {
-    if (DIR && o < 0) return side[-o - 1];
-    return p[o];
+    if (DIR && o < 0) return side ? side[-o - 1] : 0.0;
+    return HLBM_CELL_OK(o / kp.pitch, o % kp.pitch, 1, kp, SITE) ? p[o] : 0.0;
 }
 
 template <bool SIG, bool PHI0, bool DIR>
@@ -181,19 +182,20 @@ split_level_kernel(const double *F, const double *A, double *__restrict__ outA,
     }
     const double *pu = A + A_UX * P, *pv = A + A_UY * P, *pt = A + A_TH * P, *ps = A + A_S * P;
     const double rho0 = A[A_RHO * P + o], ux0 = pu[o], uy0 = pv[o], th0 = pt[o], s0 = ps[o];
+    auto at = [&](const double *p, int q, const double *side) { return plane_at<DIR, 31>(p, q, side, kp); };
     // twice the central differences
-    const double dxux = plane_at<DIR>(pu, oE, kp.d_ux) - plane_at<DIR>(pu, oW, kp.d_ux);
-    const double dyux = plane_at<DIR>(pu, oN, kp.d_ux) - plane_at<DIR>(pu, oS, kp.d_ux);
-    const double dxuy = plane_at<DIR>(pv, oE, kp.d_uy) - plane_at<DIR>(pv, oW, kp.d_uy);
-    const double dyuy = plane_at<DIR>(pv, oN, kp.d_uy) - plane_at<DIR>(pv, oS, kp.d_uy);
-    const double lap = (plane_at<DIR>(pt, oE, kp.d_th) + plane_at<DIR>(pt, oW, kp.d_th)) +
-                       (plane_at<DIR>(pt, oN, kp.d_th) + plane_at<DIR>(pt, oS, kp.d_th)) - 4.0 * th0;
+    const double dxux = at(pu, oE, kp.d_ux) - at(pu, oW, kp.d_ux);
+    const double dyux = at(pu, oN, kp.d_ux) - at(pu, oS, kp.d_ux);
+    const double dxuy = at(pv, oE, kp.d_uy) - at(pv, oW, kp.d_uy);
+    const double dyuy = at(pv, oN, kp.d_uy) - at(pv, oS, kp.d_uy);
+    const double lap = (at(pt, oE, kp.d_th) + at(pt, oW, kp.d_th)) +
+                       (at(pt, oN, kp.d_th) + at(pt, oS, kp.d_th)) - 4.0 * th0;
     // u ds/dx with limited upwind faces (muscl_adv): (s0 + d0/2) - (sq + dq/2)
     // from the upwind side q, times |u|; on the mirrored stencil of u < 0 the
     // slopes change sign.  Both sides are loaded before u is known.
     auto face = [&](double u, int om, int op, const double *pd) {
-        const double sm = plane_at<DIR>(ps, om, kp.d_s), sq = plane_at<DIR>(ps, op, kp.d_s);
-        const double dm = DIR && om < 0 ? 0.0 : pd[om], dq = DIR && op < 0 ? 0.0 : pd[op];
+        const double sm = at(ps, om, kp.d_s), sq = at(ps, op, kp.d_s);
+        const double dm = at(pd, om, nullptr), dq = at(pd, op, nullptr);  // no slope on a Dirichlet side
         const bool pos = positive64(u);
         return fma(pos ? 0.5 : -0.5, pd[o] - (pos ? dm : dq), s0 - (pos ? sm : sq));
     };
@@ -268,13 +270,14 @@ __device__ __forceinline__ void populations64(double rho, double ux, double uy, 
 }
 
 // The two limited slopes of s at a cell.
-template <bool DIR>
+template <bool DIR, int SITE>
 __device__ __forceinline__ void slopes64(const double *ps, int o, const Cross &c, const KParams &kp,
                                          const SplitPlanes &sp)
 {
     const double s0 = ps[o];
-    sp.dx[o] = va_slope64(s0 - plane_at<DIR>(ps, c.w, kp.d_s), plane_at<DIR>(ps, c.e, kp.d_s) - s0);
-    sp.dy[o] = va_slope64(s0 - plane_at<DIR>(ps, c.s, kp.d_s), plane_at<DIR>(ps, c.n, kp.d_s) - s0);
+    auto at = [&](int q) { return plane_at<DIR, SITE>(ps, q, kp.d_s, kp); };
+    sp.dx[o] = va_slope64(s0 - at(c.w), at(c.e) - s0);
+    sp.dy[o] = va_slope64(s0 - at(c.s), at(c.n) - s0);
 }
 
 // A: the auxiliary planes of level n+1 (split_level_kernel wrote s); a1 goes
@@ -293,12 +296,13 @@ split_collide_kernel(double *__restrict__ F, double *A, const SplitPlanes sp, co
     const int o = y * kp.pitch + x;
     const Cross c = cross_of(x, y, kp);
     if (!HLBM_CELL_OK(y, x, 1, kp, 32)) return;
+    auto at = [&](const double *q, int oq, const double *side) { return plane_at<DIR, 32>(q, oq, side, kp); };
     const double *pu = sp.ux, *pv = sp.uy;
     const double rho = sp.rho[o], ux = pu[o], uy = pv[o], th = sp.th[o];
-    const double dxux = plane_at<DIR>(pu, c.e, kp.d_ux) - plane_at<DIR>(pu, c.w, kp.d_ux);
-    const double dyux = plane_at<DIR>(pu, c.n, kp.d_ux) - plane_at<DIR>(pu, c.s, kp.d_ux);
-    const double dxuy = plane_at<DIR>(pv, c.e, kp.d_uy) - plane_at<DIR>(pv, c.w, kp.d_uy);
-    const double dyuy = plane_at<DIR>(pv, c.n, kp.d_uy) - plane_at<DIR>(pv, c.s, kp.d_uy);
+    const double dxux = at(pu, c.e, kp.d_ux) - at(pu, c.w, kp.d_ux);
+    const double dyux = at(pu, c.n, kp.d_ux) - at(pu, c.s, kp.d_ux);
+    const double dxuy = at(pv, c.e, kp.d_uy) - at(pv, c.w, kp.d_uy);
+    const double dyuy = at(pv, c.n, kp.d_uy) - at(pv, c.s, kp.d_uy);
     const double p = pressure64(rho, th);
     const double e2 = p * sp.half_tmg * (dxux + dyuy);
     // E1 upwind by the cell's velocity; u = 0 (or the ablation) takes the
@@ -308,8 +312,8 @@ split_collide_kernel(double *__restrict__ F, double *A, const SplitPlanes sp, co
         const bool up = positive64(u) && !cen, down = negative64(u) && !cen;
         return fma(up || down ? 1.0 : 0.5, (up ? gc : gp) - (down ? gc : gm), e2);
     };
-    const double ex = closure(ux, plane_at<DIR>(sp.gx, c.w, kp.d_gx), sp.gx[o], plane_at<DIR>(sp.gx, c.e, kp.d_gx));
-    const double ey = closure(uy, plane_at<DIR>(sp.gy, c.s, kp.d_gy), sp.gy[o], plane_at<DIR>(sp.gy, c.n, kp.d_gy));
+    const double ex = closure(ux, at(sp.gx, c.w, kp.d_gx), sp.gx[o], at(sp.gx, c.e, kp.d_gx));
+    const double ey = closure(uy, at(sp.gy, c.s, kp.d_gy), sp.gy[o], at(sp.gy, c.n, kp.d_gy));
     const double cfd = fma(-0.25, p, sp.m_half_mu);  // half of -(mu + p / 2): the differences are doubled
     const double fdxx = cfd * (dxux - dyuy), fdxy = cfd * (dyux + dxuy);
     double axx, axy, ayy;
@@ -343,7 +347,7 @@ split_collide_kernel(double *__restrict__ F, double *A, const SplitPlanes sp, co
         relaxation64(sp.two_mu, kp.mu, pressure64(r, t), omega, mp);
     }
     sp.mp[o] = mp;
-    slopes64<DIR>(A + A_S * P, o, c, kp, sp);
+    slopes64<DIR, 32>(A + A_S * P, o, c, kp, sp);
 }
 
 // What the first level pass reads beside F, s and a1, from the expressions of
@@ -359,6 +363,7 @@ split_prepare_kernel(const double *__restrict__ F, double *A, const SplitPlanes 
     if (x >= kp.nx || y >= kp.ny) return;
     const long long P = kp.plane;
     const int o = y * kp.pitch + x;
+    if (!HLBM_CELL_OK(y, x, 1, kp, 33)) return;
     double r, t;
     if (DERIVE) {
         double f[9], u, v;
@@ -376,7 +381,7 @@ split_prepare_kernel(const double *__restrict__ F, double *A, const SplitPlanes 
     double omega, mp;
     relaxation64(sp.two_mu, kp.mu, pressure64(r, t), omega, mp);
     sp.mp[o] = mp;
-    slopes64<DIR>(A + A_S * P, o, cross_of(x, y, kp), kp, sp);
+    slopes64<DIR, 33>(A + A_S * P, o, cross_of(x, y, kp), kp, sp);
 }
 
 }  // namespace hlbm
