@@ -140,9 +140,9 @@ typedef struct hlbm_handle hlbm_handle;
  * HLBM_FP64 without wall sides each copy has 4 more planes, each cell's rho,
  * u_x, u_y, theta of the level it holds (derived state: hlbm_init_fields
  * computes them, each step stores them for the next; checkpoints carry them
- * on grids above 768^2 cells and derive them again on smaller ones), and
- * the staging buffer 12 more planes for what the step's two passes hand to
- * each other.  The
+ * on grids above 768^2 cells and derive them again on smaller ones); what
+ * the step's two passes hand to each other lies in the copy that does not
+ * hold the current level and in the staging buffer.  The
  * parameters are checked before any CUDA call: HLBM_ERR_ARG for grids
  * outside 1 .. 2^28 cells or values outside the ranges above (a periodic
  * side without a periodic partner included), HLBM_ERR_UNSUPPORTED for an

@@ -29,6 +29,7 @@ namespace {
 
 constexpr int kSms = 152;  // SMs of a GB300 (work is cut for them; any count is correct)
 constexpr int DIAG_BLOCKS = 2 * 152;
+constexpr long long kMarchMinCells = 768ll * 768ll;  // GB300 sweep: tiled faster up to 768^2, marching at 1024^2
 constexpr uint64_t STATE_MAGIC = 0x31305453424c4848ull;  // "HHLBST01"
 
 struct StateHeader {
@@ -59,7 +60,7 @@ struct hlbm_handle {
     size_t plane = 0;         // elements per plane
     void *state[2] = {nullptr, nullptr};
     int cur = 0;
-    double *staging = nullptr;  // 9 FP64 planes of nx*ny
+    double *staging = nullptr;  // 9 FP64 planes of nx*ny (FP64 two-pass form: staging_doubles())
     double *diag_partial = nullptr;
     double *diag_out = nullptr;
     KParams kp;
@@ -74,7 +75,6 @@ struct hlbm_handle {
     bool periodic = false;      // all four sides periodic and ny >= 4 (specialised marching kernels)
     bool mcache = false;        // FP64 marching and two-pass forms: level-n rho, u, theta planes behind the state (A_RHO .. A_TH)
     bool split = false;         // FP64 two-pass form (hlbm_split.cuh)
-    double *split_buf = nullptr;  // its planes between the passes, behind the staging planes
     void *wall_g = nullptr;     // wall ghost rows (KParams::wall_g)
     int march_nseg = 1;         // row segments per strip
     int *d_err = nullptr;       // device-side timeout flag of the TMA kernel
@@ -168,16 +168,32 @@ static void split_shape(const hlbm_handle *h, dim3 *grid, dim3 *blk)
     *grid = dim3((h->p.nx + 31) / 32, (h->p.ny + rows - 1) / rows);
 }
 
-// outA: the auxiliary planes the step writes.
-static SplitPlanes split_planes(const hlbm_handle *h, double *outA)
+// Doubles of the staging buffer: nine planes of caller fields, or as many
+// padded planes as the two passes hand on in it, if those take more.
+static size_t staging_doubles(const hlbm_params &p, size_t plane, bool two_pass)
 {
-    double *b = h->split_buf;
+    const size_t ncell = (size_t)p.nx * p.ny;
+    const size_t hand = (long long)ncell > kMarchMinCells ? SPLIT_NHAND : SPLIT_NHAND_CANON;
+    return std::max(9 * ncell, two_pass ? hand * plane : 0);
+}
+
+// slopes: the population planes of the state copy that does not hold the
+// current level.  They are free from the end of a step's level pass, which is
+// the last to read them, until the collide pass of the next step writes
+// populations there: the slopes and mu / (2 mu + p), which go from the
+// collide pass to the next level pass, live in three of them.  The planes
+// that go from the level pass to the collide pass lie in the staging buffer,
+// which other calls use between steps only.  outA: the auxiliary planes the
+// step writes.
+static SplitPlanes split_planes(const hlbm_handle *h, double *slopes, double *outA)
+{
+    double *b = h->staging;
     const size_t P = h->plane;
-    SplitPlanes sp{b, b + P, b + 2 * P, b + 3 * P, b + 4 * P, b + 5 * P, b + 6 * P, b + 7 * P,
+    SplitPlanes sp{slopes, slopes + P, slopes + 2 * P, b, b + P, b + 2 * P, b + 3 * P, b + 4 * P,
                    outA + A_RHO * P, outA + A_UX * P, outA + A_UY * P, outA + A_TH * P,
                    2.0 * h->kp.mu, -0.5 * h->kp.mu, 0.25 * h->kp.mu, 0.5 * h->kp.two_minus_gamma, 1.0 - h->kp.sigma};
     if (!h->mcache) {
-        sp.rho = b + 8 * P; sp.ux = b + 9 * P; sp.uy = b + 10 * P; sp.th = b + 11 * P;
+        sp.rho = b + 5 * P; sp.ux = b + 6 * P; sp.uy = b + 7 * P; sp.th = b + 8 * P;
     }
     return sp;
 }
@@ -198,7 +214,7 @@ static cudaError_t split_prepare(hlbm_handle *h, bool derive)
     split_shape(h, &grid, &blk);
     const double *F = pop_planes<double, FullStore<double>>(h, h->cur);
     double *A = aux_planes<double, FullStore<double>>(h, h->cur);
-    const SplitPlanes sp = split_planes(h, A);
+    const SplitPlanes sp = split_planes(h, pop_planes<double, FullStore<double>>(h, h->cur ^ 1), A);
     if (any_dirichlet(h)) {
         if (derive) split_prepare_kernel<true, true><<<grid, blk, 0, h->stream>>>(F, A, sp, h->kp);
         else split_prepare_kernel<true, false><<<grid, blk, 0, h->stream>>>(F, A, sp, h->kp);
@@ -216,12 +232,12 @@ static cudaError_t launch_split_t(hlbm_handle *h)
     split_shape(h, &grid, &blk);
     const int a = h->cur, b = h->cur ^ 1;
     using S = FullStore<double>;
-    double *outF = pop_planes<double, S>(h, b), *outA = aux_planes<double, S>(h, b);
-    const SplitPlanes sp = split_planes(h, outA);
-    const cudaError_t e = launch_chained(split_level_kernel<SIG, PHI0, DIR>, grid, blk, 0, h->stream,
-                                         (const double *)pop_planes<double, S>(h, a), (const double *)aux_planes<double, S>(h, a),
-                                         outA, sp, h->kp);
+    double *inF = pop_planes<double, S>(h, a), *outF = pop_planes<double, S>(h, b), *outA = aux_planes<double, S>(h, b);
+    SplitPlanes sp = split_planes(h, outF, outA);
+    const cudaError_t e = launch_chained(split_level_kernel<SIG, PHI0, DIR>, grid, blk, 0, h->stream, (const double *)inF,
+                                         (const double *)aux_planes<double, S>(h, a), outA, sp, h->kp);
     if (e != cudaSuccess) return e;
+    sp = split_planes(h, inF, outA);  // what the collide pass leaves for the next level pass
     if (h->mcache) return launch_chained(split_collide_kernel<SIG, DIR, false>, grid, blk, 0, h->stream, outF, outA, sp, h->kp);
     return launch_chained(split_collide_kernel<SIG, DIR, true>, grid, blk, 0, h->stream, outF, outA, sp, h->kp);
 }
@@ -384,7 +400,6 @@ static cudaError_t launch_tma(hlbm_handle *h)
 constexpr int kNumMarch = 4;
 constexpr int kMarchMinRows = 8;
 constexpr int kMarchMaxRows = 32;
-constexpr long long kMarchMinCells = 768ll * 768ll;  // GB300 sweep: tiled faster up to 768^2, marching at 1024^2
 
 // Row segments per strip: the fewest whole waves of resident CTAs (per_sm x
 // SMs) whose segments are at most kMarchMaxRows high, cut as finely as that
@@ -775,9 +790,8 @@ int hlbm_create(const hlbm_params *params, void *stream, hlbm_handle **out)
     for (int k = 0; k < 4; k++) wall_side = wall_side || params->bc[k] == HLBM_BC_WALL;
     h->mcache = params->precision == HLBM_FP64 && !wall_side;
     const size_t bytes = alloc_bytes(h);
-    const size_t ncell = (size_t)params->nx * params->ny;
     const bool two_pass = h->mcache && !getenv("HLBM_MARCH");
-    const size_t staging = 9 * ncell + (two_pass ? SPLIT_NPLANE_CANON * h->plane + 16 : 0);
+    const size_t staging = staging_doubles(*params, h->plane, two_pass);
     if (cudaMalloc(&h->state[0], bytes) != cudaSuccess || cudaMalloc(&h->state[1], bytes) != cudaSuccess ||
         cudaMalloc(&h->staging, staging * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&h->diag_partial, DIAG_BLOCKS * DIAG_NV * sizeof(double)) != cudaSuccess ||
@@ -845,7 +859,6 @@ int hlbm_create(const hlbm_params *params, void *stream, hlbm_handle **out)
         // checkpoints carry the cache planes on the grids whose marching form
         // does, and hold 13 planes on smaller ones, as with the tiled kernel
         h->mcache = (long long)params->nx * params->ny > kMarchMinCells;
-        h->split_buf = h->staging + (9 * ncell + 15) / 16 * 16;
         *out = h;
         return HLBM_OK;
     }

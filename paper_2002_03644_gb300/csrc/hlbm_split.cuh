@@ -54,7 +54,8 @@ struct SplitPlanes {
     // constants of the case that would each cost an FP64 instruction per cell
     double two_mu, m_half_mu, quarter_mu, half_tmg, one_m_sigma;
 };
-constexpr int SPLIT_NPLANE = 8, SPLIT_NPLANE_CANON = 12;
+// planes that go from the level pass to the collide pass
+constexpr int SPLIT_NHAND = 5, SPLIT_NHAND_CANON = 9;
 
 // x > 0 and x < 0, false for NaN as the comparisons are, on the integer pipe (a
 // comparison of doubles takes the FP64 pipe like a multiply-add): the bits of
