@@ -490,17 +490,19 @@ wgrad_mma_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__res
             }
 }
 
-// The same sums with all nine taps in one CTA, for images of KT columns where
-// a chunk is whole image rows.  wgrad_mma_kernel reads dz and h once per tap,
+// The same sums with all nine taps in one CTA, for images whose rows are cut
+// into segments of KT columns: a chunk is 16384 / KT rows of a segment, down
+// the images.  wgrad_mma_kernel reads dz and h once per tap,
 // and at 8 x 256^2 those 1.2 GB per 64 -> 64 layer come from L2 at 4.6 TB/s
 // (262 us).  Here a CTA takes 16 input and COB output channels
-// of a chunk: one image row of dz at a time against the three rows of h its
+// of a chunk: one segment row of dz at a time against the three rows of h its
 // taps reach (a ring of four row slots, the next row copied while this one
 // is computed), 96 or 128 bytes per pixel instead of nine times 256.  Warp
 // (dp, m) holds the three taps of row offset dp (a dz fragment serves three
 // taps); two more warps only copy, so that the address arithmetic of the
-// copies does not stand in the chains of the products.  The chain of a result runs over the chunk's pixels in the same
-// order as in wgrad_mma_kernel, so both give the same bits.  At 8 x 256^2 the
+// copies does not stand in the chains of the products.  The chain of a result runs over 16384 pixels as in
+// wgrad_mma_kernel, and with one segment per row over the same ones in the
+// same order, so both give the same bits then.  At 8 x 256^2 the
 // 64 -> 64 layer takes 128 us, 300 TFLOP/s: 256 CTAs, two per SM, bound by
 // their ldmatrix reads of shared memory (four per six MMAs, 12 warps: 192
 // cycles per 16-pixel step).
@@ -517,7 +519,7 @@ struct WgRowGeom {
 // grid: (chunk, block of COB output channels, block of 16 input channels)
 template <int CIN, int COUT, int KT>
 __global__ void __launch_bounds__(WgRowGeom<COUT, KT>::THREADS)
-wgrad_rows_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ dzb, int nrow, int H,
+wgrad_rows_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__restrict__ dzb, int nrow, int H, int W,
                   float *__restrict__ part)
 {
     using G = WgRowGeom<COUT, KT>;
@@ -531,17 +533,24 @@ wgrad_rows_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__re
     const int dp = warp % 3, m0 = warp / 3 * 16;
     const bool copier = warp >= G::MMA_WARPS;
     const int ct = threadIdx.x - 32 * G::MMA_WARPS;
-    const int r0 = blockIdx.x * (WG_CHUNK / KT), r1 = min(r0 + WG_CHUNK / KT, nrow);  // image rows n H + i
-    auto load_h = [&](int row, int slot) {  // pixels -1 .. KT (wrapped) of an image row
-        const __nv_bfloat16 *src = h + (size_t)row * KT * CIN + c0;
+    // rows are numbered column segment first: seg nrow + (n H + i); first: the
+    // segment's row 0 of the first image, j0 its first column
+    const int r0 = blockIdx.x * (WG_CHUNK / KT), r1 = min(r0 + WG_CHUNK / KT, W / KT * nrow);
+    int j0 = r0 / nrow * KT, first = r0 / nrow * nrow;
+    auto load_h = [&](int row, int slot) {  // pixels -1 .. KT of the segment (the halo its neighbours', wrapped)
+        const __nv_bfloat16 *src = h + ((size_t)(row - first) * W + j0) * CIN + c0;
         __nv_bfloat16 *dst = sH + slot * G::H_SLOT;
         for (int e = ct; e < (KT + 2) * 2; e += G::COPIERS) {
             const int px = e >> 1, c8 = e & 1;
-            cp_async16(dst + px * LDB + c8 * 8, src + (size_t)((px + KT - 1) % KT) * CIN + c8 * 8);
+            int j = px - 1;
+            if (px == 0 && j0 == 0) j = W - 1;
+            if (px == KT + 1 && j0 + KT == W) j = -j0;
+            cp_async16(dst + px * LDB + c8 * 8, src + (ptrdiff_t)j * CIN + c8 * 8);
         }
     };
     auto load_z = [&](int row, int buf) {
-        const __nv_bfloat16 *src = dzb + (size_t)row * KT * COUT + o0;
+        const bool next = row - first == nrow;  // the next segment's first row
+        const __nv_bfloat16 *src = dzb + ((size_t)(next ? 0 : row - first) * W + j0 + (next ? KT : 0)) * COUT + o0;
         __nv_bfloat16 *dst = sZ + buf * G::Z_SLOT;
         for (int e = ct; e < KT * CA; e += G::COPIERS) {
             const int px = e / CA, c8 = e - px * CA;
@@ -560,6 +569,7 @@ wgrad_rows_kernel(const __nv_bfloat16 *__restrict__ h, const __nv_bfloat16 *__re
     for (int row = r0; row < r1; row++) {
         const int buf = (row - r0) & 1;
         const bool more = row + 1 < r1, same = i + 1 < H;
+        if (row - first == nrow) { first += nrow; j0 += KT; }
         if (row == r0 || i == 0) base = 0;
         if (copier) {
             if (row == r0 || i == 0) {
@@ -713,22 +723,36 @@ cudaError_t launch_wgrad_rows(const WgradArgs &a, cudaStream_t st)
     if (e != cudaSuccess) return e;
     const int chunks = (a.npix + WG_CHUNK - 1) / WG_CHUNK;
     wgrad_rows_kernel<CIN, COUT, KT><<<dim3(chunks, COUT / G::COB, CIN / 16), G::THREADS, G::smem_bytes, st>>>(
-        a.h, a.dzb, a.npix / KT, a.H, a.part);
+        a.h, a.dzb, a.npix / a.W, a.H, a.W, a.part);
     wgrad_reduce_kernel<<<(9 * CIN * COUT + 31) / 32, 256, 0, st>>>(a.part, chunks, a.cout, a.cin, COUT, CIN, a.dW);
     return cudaGetLastError();
 }
 
-// Images of 256 columns take the kernel with all taps per CTA (64 -> 64
-// channels, 8 / 4 / 1 images: 128 / 80 / 79 us against 262 / 158 / 95 us for
-// one CTA per tap; with 128 columns it was no faster, 118 against 102 us,
-// because a row is then only 8 of its steps).  Elsewhere one CTA per (chunk,
-// tap) takes all input channels where that gives 1.5 CTAs per SM, else
-// blocks of fewer channels (8 images of 128^2: 102 us).
+// Widths that are cut into segments of 256 columns take the kernel with all
+// taps per CTA, from a number of chunks that depends on the channels: with
+// few channels a chunk is few CTAs (COUT / 32 x CIN / 16; one CTA per tap and
+// chunk gives nine).  A backward pass of four layers, one CTA per tap against
+// all taps (us; what decides is the pixels, not whether a row is one segment
+// or five):
+//   64 -> 64   1 x 64 x 256 534, 511;  1 x 100 x 1280 747, 724;  1 x 512^2 1201, 966;
+//              8 x 256^2 2101, 1580;  2 x 512^2 2082, 1578;  16 x 256^2 4035, 3023
+//   48 -> 48   1 x 64 x 256 523, 463;  2 x 512^2 1960, 1498
+//   16 <-> 64  1 x 64 x 256 439, 437;  1 x 512^2 672, 563;  2 x 512^2 967, 707
+//   32 <-> 64  8 chunks (2 x 256^2) 715, 720;  16 chunks (1 x 512^2) 982, 927
+//   32 -> 32   16 chunks 759, 797;  32 chunks (2 x 512^2) 1244, 1144
+//   16 -> 16   16 chunks 469, 477;  32 chunks 565, 558
+// Segments of 128 columns would give shorter rows of work between barriers: 64
+// -> 64 (six layers) 1002 against 807 per tap at 8 x 128^2, though 1330 against
+// 1850 at 32 x 128^2 and 1401 against 2728 at 4 x 384^2, which are left to the
+// per-tap kernel.  That one takes all input channels per CTA where that gives
+// 1.5 CTAs per SM, else blocks of fewer channels.
 template <int CIN, int COUT>
 cudaError_t launch_wgrad_t(const WgradArgs &a, cudaStream_t st)
 {
-    if (a.W == 256) return launch_wgrad_rows<CIN, COUT, 256>(a, st);
     const long long chunks = (a.npix + WG_CHUNK - 1) / WG_CHUNK, sms = sm_count();
+    constexpr bool wide = CIN > 32 || COUT > 32;
+    constexpr int least = !wide ? 32 : (CIN == 32 || COUT == 32 ? 16 : 1);
+    if (a.W % 256 == 0 && chunks >= least) return launch_wgrad_rows<CIN, COUT, 256>(a, st);
     const long long ctas = 9 * chunks, want = 3 * sms / 2;
     if constexpr (CIN == 64) {
         if (ctas < want) return 2 * ctas < want ? launch_wgrad_block<CIN, COUT, 16>(a, st) : launch_wgrad_block<CIN, COUT, 32>(a, st);
