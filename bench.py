@@ -235,7 +235,7 @@ def measured_peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("hlbm_device.cuh", "hlbm_tma.cuh", "hlbm_march.cuh", "hlbm_pack.cuh", "hlbm_api.cu"):
+    for f in ("hlbm_device.cuh", "hlbm_tma.cuh", "hlbm_march.cuh", "hlbm_split.cuh", "hlbm_tables64.h", "hlbm_pack.cuh", "hlbm_api.cu"):
         h.update(open(os.path.join(ROOT, "paper_2002_03644_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
