@@ -494,12 +494,12 @@ static cudaError_t march_dispatch(hlbm_handle *h)
 
 static cudaError_t setup_march(hlbm_handle *h)
 {
-    // Every precision marches by default on grids of more than
+    // The FP32-arithmetic forms march by default on grids of more than
     // kMarchMinCells cells (below that a grid has too few strips and
-    // segments to fill the GPU, and the tiled kernel is faster).  In FP64 the
-    // marching kernel is 2-8 % faster at 1024^2-2048^2: it recomputes less
-    // halo on the FP64 pipe.  HLBM_MARCH=<k> picks a variant, -1 the tiled /
-    // TMA kernels.
+    // segments to fill the GPU, and the tiled kernel is faster).
+    // HLBM_MARCH=<k> picks a variant, -1 the tiled / TMA kernels; FP64 comes
+    // here only with HLBM_MARCH set (its marching kernel takes 764 us per step
+    // at 1024^2, its tiled one 951, the two-pass form 369).
     const bool big = (long long)h->p.nx * h->p.ny > kMarchMinCells;
     h->march_variant = env_choice("HLBM_MARCH", big ? 0 : -1, -1, kNumMarch);
     if (h->march_variant < 0) return cudaSuccess;
@@ -849,7 +849,7 @@ int hlbm_create(const hlbm_params *params, void *stream, hlbm_handle **out)
         *out = h;
         return HLBM_OK;
     }
-    // FP64: the two-pass form at every size (1024^2 vortex 377 us per step
+    // FP64: the two-pass form at every size (1024^2 vortex 369 us per step
     // against 764 on the marching kernel; Sod tube 400 x 4 13 us against 39
     // on the tiled kernel).  HLBM_MARCH=<k> picks a marching variant, -1 the
     // tiled kernel, as for the other precisions.

@@ -325,9 +325,11 @@ __device__ __forceinline__ float ex2_approx(float x)
 //   exp: x = (128 n + j) log 2 / 128 + r, |r| < 2^-8.5, exp x = 2^n 2^(j/128) e^r.
 // The truncated series leave 2^-59 and 2^-60 relative; against 64-bit mantissas
 // the largest errors found are 1.4 and 0.51 ulp (2 10^7 points per range, 64-bit
-// mantissas).  theta itself, whose exponent is rounded before the exponential,
-// is off by 3.1e-16 relative at most and 1.07e-16 rms for rho in 0.9 .. 1.1 and
-// theta in 0.15 .. 0.25, the same figures as with correctly rounded functions.  Operands outside the normal range take CUDA's functions.
+// mantissas; tests/test_gpu_fp64_functions.py holds 1.6 and 0.52).  theta
+// itself, whose exponent is rounded before the exponential, is off by 3.1e-16
+// relative at most and 1.07e-16 rms for rho in 0.9 .. 1.1 and theta in 0.15 ..
+// 0.25, the same figures as with correctly rounded functions.  Operands
+// outside the normal range take CUDA's functions.
 //
 // The tables are copied to shared memory at the start of a pass, so that a
 // lookup, which stands in the chain of dependent operations, is no trip to L2.

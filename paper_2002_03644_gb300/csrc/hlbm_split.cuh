@@ -14,18 +14,26 @@
 //   collide pass  (split_collide_kernel)  E1, E2, a1 and the collision (eqs
 //                 Psialgo, Equilibrium, a1sigalgo, streamalgo) from level n+1 of
 //                 the cell and its neighbours, and for the next level pass the
-//                 cell's two Van Albada slopes of s(n+1) and 1 / (2 mu + p).
+//                 cell's two Van Albada slopes of s(n+1) and mu / (2 mu + p).
 // A face of the MUSCL scheme needs the slopes of the cell and of its upwind
 // neighbour only, so two slopes per cell serve what took four per cell, and
-// the reciprocal serves omega (eq. streamalgo) and the Phi of the next level
-// (eq. viscous heat discret).  That leaves six reciprocals per cell-update
-// instead of eight divisions.
+// one reciprocal serves omega (eq. streamalgo) and the Phi of the next level
+// (eq. viscous heat discret).  That leaves five reciprocals per cell-update
+// (1 / (rho theta), 1 / rho, 1 / (2 mu + p) and the slopes' two) instead of
+// eight divisions.
 //
-// Measured on GB300, per step: 1024^2 vortex 377 us (764 on the marching
-// kernel), Sod tube 400 x 4 13 us (39 on the tiled kernel).  The FP64 pipe is
-// busy for 84 % of the level and the collide pass's cycles, which is what 19
-// cycles per warp instruction, the most that eight warps of dependent
-// multiply-adds reach, come to.
+// Measured on GB300, per step: 1024^2 vortex 369 us (764 on the marching
+// kernel), Sod tube 400 x 4 13 us (39 on the tiled kernel).  The level pass
+// takes 83 FP64 instructions per cell, the collide pass 92.5; the FP64 pipe is
+// busy for 85 and 86 % of their cycles, which is what 19 cycles per warp
+// instruction, the most that eight warps of dependent multiply-adds reach,
+// come to.
+//
+// Against the time step in 80-bit arithmetic (13 cases of 700 to 10000 cells,
+// all sides but walls, sigma 0 to 0.9): after one step the rms errors of rho,
+// u, theta, s and a1 are 0.997 to 1.000 times (geometric mean) those of the
+// tiled and the marching kernel with IEEE divisions and CUDA's functions;
+// after 10 to 40 steps 0.88 to 1.07 times in every smooth case.
 //
 // CANON (grids of up to 768^2 cells, whose checkpoints hold the 13 planes of
 // the tiled kernel): the cache planes a level pass reads are derived from
@@ -352,8 +360,8 @@ split_collide_kernel(double *__restrict__ F, double *A, const SplitPlanes sp, co
 }
 
 // What the first level pass reads beside F, s and a1, from the expressions of
-// the collide pass, after init or a checkpoint set the state: the slopes, the
-// reciprocals, and (DERIVE) the cache planes.
+// the collide pass, after init or a checkpoint set the state: the slopes,
+// mu / (2 mu + p), and (DERIVE) the cache planes.
 template <bool DIR, bool DERIVE>
 __global__ void __launch_bounds__(256)
 split_prepare_kernel(const double *__restrict__ F, double *A, const SplitPlanes sp, const KParams kp)

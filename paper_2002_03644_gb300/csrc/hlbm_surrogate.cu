@@ -8,11 +8,14 @@
 // arranged for the tensor-core B operand: Wb[tap][co][ci] (forward) and
 // Wd[tap][ci][co] (input gradient, read with the negated offset of the tap).
 //
-// Convolution = implicit GEMM on the BF16 tensor cores (mma.sync m16n8k16,
-// FP32 accumulators): out[pixel, n] = sum_tap sum_k B[tap][n][k] *
-// in[pixel + offset(tap), k].  One warp computes 16 pixels x 64 outputs; the
-// epilogue adds the bias and, where the layer has one, applies GELU and
-// keeps the pre-activation for the backward pass.
+// Convolution = implicit GEMM on the BF16 tensor cores with FP32
+// accumulators: out[pixel, n] = sum_tap sum_k B[tap][n][k] *
+// in[pixel + offset(tap), k].  Layers with 16 or 64 padded channels each way
+// on images whose width is a multiple of 128 take tcgen05.mma with TMEM
+// accumulators (conv_tc_kernel), other layers on such images
+// mma.sync m16n8k16 with staged rows (conv_staged_kernel), other widths
+// conv_mma_kernel.  The epilogue adds the bias and, where the layer has one,
+// applies GELU and keeps the pre-activation for the backward pass.
 //
 // Weight gradient: dW[co][ci][tap] = sum_pixels dz[pixel, co] *
 // h[pixel + offset(tap), ci], a GEMM over pixels on the tensor cores
@@ -842,7 +845,6 @@ __global__ void pack_input_kernel(const float *__restrict__ x, int c_real, int c
     }
 }
 
-// FP32 [n] -> BF16 [n]
 // dz_last[p][c] += dy[p][c] for c < c_real: an upstream gradient (from a
 // later call of a rollout through the network) added to dL/dy.
 __global__ void add_upstream_kernel(float *__restrict__ dz_last, int cpad_last, const float *__restrict__ dy,
@@ -866,6 +868,7 @@ __global__ void gather_grad_kernel(const float *__restrict__ g, int cpad, int c_
     }
 }
 
+// FP32 [n] -> BF16 [n]
 __global__ void to_bf16_kernel(const float *__restrict__ x, long long n, __nv_bfloat16 *__restrict__ out)
 {
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -1047,7 +1050,7 @@ conv_staged_kernel(const __nv_bfloat16 *__restrict__ in, const __nv_bfloat16 *__
 // ---- 5th-generation tensor cores (tcgen05, TMEM accumulators) ---------------------
 // The convolutions with CIN, NOUT in {16, 64} (padded channels) on images
 // whose width is a multiple of 128, as a persistent kernel with one CTA of
-// 17 warps per SM:
+// 19 warps per SM:
 //   - the nine taps' weights stay in shared memory for the whole launch;
 //   - each 128-pixel row segment is one M = 128 tile; a CTA walks down a
 //     contiguous run of tiles of one column segment, so consecutive tiles
