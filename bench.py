@@ -281,32 +281,17 @@ def kernel_name(precision, cells, sigma=0.0, phi_mode=0, periodic=False):
 FP64_NOMINAL_TFLOPS = 1.25
 
 
-def profiled_fp64_counts(n):
-    """FP64 operations (add, mul, 2 per fma) and FP64 instructions per
-    cell-update of the FP64 fused kernel from the committed ncu count, if it
-    was taken on the current kernel source; (None, None) otherwise."""
+def profiled(precision, n, kernel):
+    """The committed ncu summary of this kernel on the n^2 vortex, if it was
+    taken on the current kernel source; an empty dict otherwise."""
     path = os.path.join(ROOT, "profiles", "fused_step_vortex_traffic.json")
     try:
-        e = json.load(open(path)).get(f"fp64_{n}")
+        e = json.load(open(path)).get(f"{precision}_{n}")
     except Exception:
-        return None, None
-    if not e or e.get("kernel_source_hash") != kernel_source_hash():
-        return None, None
-    return e.get("fp64_flops_per_cell"), e.get("fp64_instructions_per_cell")
-
-
-def profiled_traffic(precision, n):
-    """dram bytes per launch of the fused kernel from the committed ncu
-    summary, if it was taken on the current kernel source."""
-    path = os.path.join(ROOT, "profiles", "fused_step_vortex_traffic.json")
-    try:
-        d = json.load(open(path))
-    except Exception:
-        return None
-    e = d.get(f"{precision}_{n}")
-    if not e or e.get("kernel_source_hash") != kernel_source_hash():
-        return None
-    return e.get("dram_bytes_per_launch")
+        return {}
+    if not e or e.get("kernel") != kernel or e.get("kernel_source_hash") != kernel_source_hash():
+        return {}
+    return e
 
 
 # ---- CPU oracle timing -----------------------------------------------------------------
@@ -486,15 +471,16 @@ def run_ours(args):
     bpc = bytes_per_cell(args.precision, cells)
     mean_launch_s = statistics.mean(step_ms) / 1e3
     achieved = bpc * cells / mean_launch_s / 1e9
+    kernel = kernel_name(args.precision, cells, case.sigma, case.phi_mode,
+                         all(b == 0 for b in case.bc) and case.ny >= 4
+                         and os.environ.get("HLBM_MARCH_GENERAL", "0") != "1")
+    counters = profiled(args.precision, args.n, kernel) if args.workload == "vortex" else {}
     if args.precision != "fp64":
         peak = peaks["hbm_gbs"] if peaks else 6800.0
         roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": profiled_traffic(args.precision, args.n) if args.workload == "vortex" else None,
+                "frac": achieved / peak, "traffic": counters.get("dram_bytes_per_launch"),
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback",
-                "kernel": kernel_name(args.precision, cells, case.sigma, case.phi_mode,
-                                      all(b == 0 for b in case.bc) and case.ny >= 4
-                                      and os.environ.get("HLBM_MARCH_GENERAL", "0") != "1"),
-                "algorithmic_bytes_per_launch": bpc * cells}
+                "kernel": kernel, "algorithmic_bytes_per_launch": bpc * cells}
     else:
         # FP64 is bound by GB300's FP64 pipe: FP64 operations (add, mul, 2 per
         # fma) executed per cell-update, counted by ncu, against this GPU's
@@ -502,17 +488,17 @@ def run_ours(args):
         # An add or a multiply occupies the pipe like an FMA but counts one
         # flop, so the FP64 instruction rate against the probe's FMA rate
         # (pipe_instruction_frac) is the tighter measure.
-        fpc, ipc = profiled_fp64_counts(args.n)
+        fpc, ipc = counters.get("fp64_flops_per_cell"), counters.get("fp64_instructions_per_cell")
         tf = None if fpc is None else fpc * cells / mean_launch_s / 1e12
         peak = 2.0 * fp64_fma_rate / 1e12
         roof = {"bound": "alu", "achieved": tf, "peak": peak, "unit": "TFLOP/s",
                 "frac": None if tf is None else tf / peak,
                 "pipe_instruction_frac": None if ipc is None else ipc * cells / mean_launch_s / fp64_fma_rate,
-                "traffic": profiled_traffic(args.precision, args.n) if args.workload == "vortex" else None,
+                "traffic": counters.get("dram_bytes_per_launch"),
                 "peak_source": "measured in this run: hlbm_selftest_fp64_rate, FP64 FMA chains on every SM "
                                f"(nominal {FP64_NOMINAL_TFLOPS} TFLOP/s)",
                 "fp64_flops_per_cell": fpc, "fp64_instructions_per_cell": ipc, "hbm_gbs_achieved": achieved,
-                "kernel": kernel_name(args.precision, cells, case.sigma, case.phi_mode),
+                "kernel": kernel,
                 "algorithmic_bytes_per_launch": bpc * cells}
 
     cpu = None
